@@ -145,11 +145,17 @@ def _ptr(x):
     return x.data_ptr()
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise RuntimeError("lbtracer needs a CUDA device; there is no CPU fallback")
-    return torch
+    global _torch_module
+    if _torch_module is None:  # a device once found stays: asking the driver takes longer than a small launch
+        import torch
+        if not torch.cuda.is_available():
+            raise RuntimeError("lbtracer needs a CUDA device; there is no CPU fallback")
+        _torch_module = torch
+    return _torch_module
 
 
 def box_desc(E, tau, periodic=(False, False, False), time_interp=LB_TIME_LINEAR, K=1, nbeads=0, rho_b=1.0,
@@ -203,6 +209,8 @@ class Tracers:
         nbytes = _sz()
         _check(lib.lb_plan(arr, len(self.descs), storage, int(ring_slots), ctypes.byref(nbytes)))
         self.stream = stream if stream is not None else torch.cuda.Stream()
+        self._device, self._raw_stream = self.stream.device.index, self.stream.cuda_stream
+        self._current_raw = torch._C._cuda_getCurrentRawStream
         self.arena = torch.empty(int(nbytes.value), dtype=torch.uint8, device=self.stream.device)
         # the arena may reuse memory that work still pending on torch's current
         # stream reads; the context's own stream must come after that work
@@ -219,11 +227,11 @@ class Tracers:
         current stream when device memory that stream produced (or last used)
         is handed to the library: torch enqueues on its current stream, the
         library on the context's stream."""
+        if self._current_raw(self._device) == self._raw_stream:  # the common case of a caller on the context's stream
+            return
         if tensors and not any(getattr(t, "is_cuda", False) for t in tensors):
             return
-        cur = self.torch.cuda.current_stream(self.stream.device)
-        if cur != self.stream:
-            self.stream.wait_stream(cur)
+        self.stream.wait_stream(self.torch.cuda.current_stream(self.stream.device))
 
     # ---- thin wrappers (same names as the C ABI) ----
     def lb_init(self, box, u0):
