@@ -117,7 +117,7 @@ Layout plan_layout(const lb_box_desc* boxes, int nboxes, int storage, int ring_s
             zst = align_up(zst + 6 * 3 * Ec * Ec * real_bytes(storage));
         }
         beads += boxes[b].nbeads;
-        const int64_t c = (n3 + 4095) / 4096;
+        const int64_t c = (n3 + kConsChunk - 1) / kConsChunk;
         if (c > chunks) chunks = c;
     }
     L.pop_bytes = pop;

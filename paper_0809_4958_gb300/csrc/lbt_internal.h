@@ -60,6 +60,8 @@ __host__ __device__ inline void frame_accel_at(const BoxDev& bd, const double* f
     for (int c = 0; c < 3; c++) a[c] += (1.0 - th) * a0[c] + th * a1[c];
 }
 
+constexpr int64_t kConsChunk = 2048;  // sites one block of the conservation sums takes
+
 constexpr double kBeadSkin = 0.3;  // Verlet skin of the bead pair lists (lattice units)
 
 // Indices of the per-chain MD constants (ChainDev::md_d / md_f).

@@ -1428,13 +1428,85 @@ __global__ void k_read_dev(const typename Stor<ST>::E* Ab, int64_t count, typena
         dst[s] = (typename Stor<ST>::R)Stor<ST>::in(Ab[s]);
 }
 
+// Density deviation and (WHAT = 1) momentum of one site from its populations,
+// by opposite pairs: their sums make the density, their differences the
+// momentum (39 additions in place of 48).
+template <class A, int WHAT, class F>
+__device__ __forceinline__ void site_moments(const F& f, A& r, A j[3])
+{
+    r = f(0);
+#pragma unroll
+    for (int i = 1; i < kQ; i += 2) {
+        const A a = f(i), b = f(i + 1);
+        r += a + b;
+        if (WHAT == 1) {
+            const A d = a - b;
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                if (i == 1 + 2 * c) j[c] = d;  // the axis pairs come first
+                else if (cvec(i, c) > 0) j[c] += d;
+                else if (cvec(i, c) < 0) j[c] -= d;
+            }
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Conservation sums in FP64: block (chunk, box) sums its sites into a partial,
-// then one thread per box adds the partials in chunk order.
+// then one block per box adds the partials in a fixed order.
+//
+// One read of the populations.  The FP64 pipe runs two lanes a clock, so 57
+// additions and 19 conversions a site bounded the sweep (328 us for a 128^3
+// FP32 box whose bytes take 23 us).  The populations of the reduced formats
+// are FP32 values: a thread now sums them exactly enough in FP32 alone, as an
+// unevaluated sum of three words (each addition splits off its rounding error,
+// two levels deep, 72 bits in all, more than the 53 of an FP64 sum), two
+// adjacent sites to an instruction, and converts once at the end: 79 us, bound
+// by those additions.  A block of 128 threads takes 2048 sites, so that a 128^3 box has seven blocks
+// to an SM rather than three or four.
 // ---------------------------------------------------------------------------
-constexpr int kConsThreads = 256;
-constexpr int kConsSitesPerThread = 16;
-constexpr int64_t kConsChunk = (int64_t)kConsThreads * kConsSitesPerThread;
+constexpr int kConsThreads = 128;
+constexpr int kConsSitesPerThread = kConsChunk / kConsThreads;
+
+// Sums of two streams of FP32 values as unevaluated sums s + e + f: Knuth's
+// two-sum on s, its error added to e by another two-sum, that error to f.
+struct Sum3 {
+    float2 s = {0.f, 0.f}, e = {0.f, 0.f}, f = {0.f, 0.f};
+    static __device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& err)
+    {
+        const float2 t = add2(a, b), bb = sub2(t, a);
+        err = add2(sub2(a, sub2(t, bb)), sub2(b, bb));
+        return t;
+    }
+    __device__ __forceinline__ void add(float2 x)
+    {
+        float2 r;
+        s = two_sum(s, x, r);
+        e = two_sum(e, r, r);
+        f = add2(f, r);
+    }
+    __device__ __forceinline__ double value() const
+    {
+        return ((double)s.x + ((double)e.x + (double)f.x)) + ((double)s.y + ((double)e.y + (double)f.y));
+    }
+};
+
+// Sums over this thread's sites of a chunk in FP64 (every format; the reduced
+// ones only where a value is not finite or so large that FP32 overflows).
+template <int ST>
+__device__ __noinline__ void cons_sites_f64(const typename Stor<ST>::E* Ab, int64_t c0, int64_t n3, double acc[4])
+{
+    for (int a = 0; a < 4; a++) acc[a] = 0.0;
+    for (int k = 0; k < kConsSitesPerThread / 2; k++)
+        for (int h = 0; h < 2; h++) {
+            const int64_t site = c0 + 2 * ((int64_t)k * kConsThreads + threadIdx.x) + h;
+            if (site >= n3) return;
+            double r, j[3];
+            site_moments<double, 1>([&](int i) { return (double)Stor<ST>::in(Ab[(int64_t)i * n3 + site]); }, r, j);
+            acc[0] += r;
+            for (int a = 0; a < 3; a++) acc[1 + a] += j[a];
+        }
+}
 
 template <int ST>
 __global__ void __launch_bounds__(kConsThreads) k_cons_partial(const void* Araw, const BoxDev* boxes, int64_t chunks,
@@ -1447,18 +1519,32 @@ __global__ void __launch_bounds__(kConsThreads) k_cons_partial(const void* Araw,
     const int64_t c0 = (int64_t)blockIdx.x * kConsChunk;
     if (c0 >= n3) return;
     const typename S::E* Ab = reinterpret_cast<const typename S::E*>(Araw) + bd.f_off;
-    double acc[4] = {0, 0, 0, 0};
-    for (int k = 0; k < kConsSitesPerThread; k++) {
-        const int64_t s = c0 + (int64_t)k * kConsThreads + threadIdx.x;
-        if (s >= n3) break;
+    double acc[4];
+    if constexpr (ST == kF64) {
+        cons_sites_f64<ST>(Ab, c0, n3, acc);
+    } else {
+        Sum3 t[4];
+        for (int k = 0; k < kConsSitesPerThread / 2; k++) {
+            const int64_t site = c0 + 2 * ((int64_t)k * kConsThreads + threadIdx.x);  // n3 is even
+            if (site >= n3) break;
+            float2 v[kQ];
 #pragma unroll
-        for (int i = 0; i < kQ; i++) {
-            const double d = (double)S::in(Ab[(int64_t)i * n3 + s]);
-            acc[0] += d;
-            if (cvec(i, 0)) acc[1] += cvec(i, 0) * d;
-            if (cvec(i, 1)) acc[2] += cvec(i, 1) * d;
-            if (cvec(i, 2)) acc[3] += cvec(i, 2) * d;
+            for (int i = 0; i < kQ; i++) v[i] = PairIO<ST>::even(Ab + (int64_t)i * n3, (int)site);
+#pragma unroll
+            for (int i = 0; i < kQ; i++) {
+                t[0].add(v[i]);
+#pragma unroll
+                for (int a = 0; a < 3; a++)
+                    if (cvec(i, a)) t[1 + a].add(cvec(i, a) > 0 ? v[i] : make_float2(-v[i].x, -v[i].y));
+            }
         }
+        bool finite = true;
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+            acc[a] = t[a].value();
+            finite = finite && isfinite(acc[a]);
+        }
+        if (!finite) cons_sites_f64<ST>(Ab, c0, n3, acc);
     }
     __shared__ double red[kConsThreads / 32][4];
     for (int a = 0; a < 4; a++)
@@ -1466,14 +1552,14 @@ __global__ void __launch_bounds__(kConsThreads) k_cons_partial(const void* Araw,
     if ((threadIdx.x & 31) == 0)
         for (int a = 0; a < 4; a++) red[threadIdx.x >> 5][a] = acc[a];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t[4] = {0, 0, 0, 0};
-        for (int w = 0; w < kConsThreads / 32; w++)
-            for (int a = 0; a < 4; a++) t[a] += red[w][a];
-        for (int a = 0; a < 4; a++) partial[((int64_t)b * chunks + blockIdx.x) * 4 + a] = t[a];
+    if (threadIdx.x < 4) {
+        double t = 0;
+        for (int w = 0; w < kConsThreads / 32; w++) t += red[w][threadIdx.x];
+        partial[((int64_t)b * chunks + blockIdx.x) * 4 + threadIdx.x] = t;
     }
 }
 
+constexpr int kConsFinalThreads = 256;
 __global__ void k_cons_final(const BoxDev* boxes, const ChainDev* chains, int nboxes, int64_t chunks,
                              const double* partial, const double* vel, double* out, int32_t* status);
 
@@ -1654,7 +1740,7 @@ cudaError_t Launch<ST>::conservation(const void* A, const BoxDev* boxes, const C
     k_cons_partial<ST><<<grid, kConsThreads, 0, s>>>(A, boxes, chunks, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_cons_final<<<(nboxes + 127) / 128, 128, 0, s>>>(boxes, chains, nboxes, chunks, partial, vel, out, status);
+    k_cons_final<<<nboxes, kConsFinalThreads, 0, s>>>(boxes, chains, nboxes, chunks, partial, vel, out, status);
     return cudaGetLastError();
 }
 

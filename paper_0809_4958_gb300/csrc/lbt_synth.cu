@@ -179,26 +179,69 @@ cudaError_t launch_synth_volume(const double* kvec, const double* amp, const dou
 // Each block writes the sum of its sites (grid-stride order, then a fixed
 // tree); one thread adds the block sums in order and divides by the count.
 constexpr int kVortThreads = 256;
-constexpr int kVortMaxBlocks = 512;
+constexpr int kVortMaxBlocks = 456;  // three to each of the 152 SMs; the scratch holds 512 sums
 
+// Sum over the threads of a block in a fixed order (shuffle
+// tree, then the warps in turn); every thread gets it.
+__device__ double block_sum(double v, double* sh)
+{
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += sh[w];
+    return t;
+}
+
+// An FP32 value in FP64 by moving its bits (the conversion instruction runs on
+// the FP64 pipe, two lanes a clock); zeros, subnormals, infinities and NaN
+// through the conversion itself.
+__device__ __forceinline__ double widen(float v)
+{
+    const uint32_t b = __float_as_uint(v);
+    if ((b << 1) - 0x01000000u >= 0xfe000000u) return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// sqrt(x) by Goldschmidt's iteration from an FP32 start: two steps from 22
+// bits (x outside the FP32 range, zero, infinite or NaN: the library's).
+__device__ __forceinline__ double quick_sqrt(double x)
+{
+    if (!(x > 1e-30 && x < 1e30)) return sqrt(x);
+    const double y = widen(rsqrtf(__double2float_rn(x)));
+    double g = x * y, h = 0.5 * y;
+    double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    return fma(fma(-g, g, x), h, g);
+}
+
+// Bounded by the FP64 pipe: 9 differences, 3 products and a root a site.  With
+// the library's square root and a conversion instruction per value the whole
+// interior of a 128^3 FP32 box took 146 us.
 template <class R>
 __global__ void __launch_bounds__(kVortThreads) k_vort_partial(const R* u, int E, int lo, int hi, double* partial)
 {
     const int m = hi - lo + 1;
-    const int64_t cube = (int64_t)m * m * m, n3 = (int64_t)E * E * E;
-    const int64_t sy = E, sz = (int64_t)E * E;
-    const R* ux = u;
-    const R* uy = u + n3;
-    const R* uz = u + 2 * n3;
+    const int cube = m * m * m;  // below 1024^3
+    const int64_t n3 = (int64_t)E * E * E;
+    const int sy = E, sz = E * E;
     double acc = 0.0;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < cube; s += (int64_t)gridDim.x * blockDim.x) {
-        const int x = lo + (int)(s % m), y = lo + (int)((s / m) % m), z = lo + (int)(s / ((int64_t)m * m));
-        const int64_t c = (int64_t)z * sz + (int64_t)y * sy + x;
-        const double wx = 0.5 * ((double)uz[c + sy] - (double)uz[c - sy]) - 0.5 * ((double)uy[c + sz] - (double)uy[c - sz]);
-        const double wy = 0.5 * ((double)ux[c + sz] - (double)ux[c - sz]) - 0.5 * ((double)uz[c + 1] - (double)uz[c - 1]);
-        const double wz = 0.5 * ((double)uy[c + 1] - (double)uy[c - 1]) - 0.5 * ((double)ux[c + sy] - (double)ux[c - sy]);
-        acc += sqrt(wx * wx + wy * wy + wz * wz);
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < cube; s += gridDim.x * blockDim.x) {
+        const int row = s / m, zz = row / m;
+        const int x = lo + s - row * m, y = lo + row - zz * m, z = lo + zz;
+        const R* ux = u + ((int64_t)z * sz + y * sy + x);
+        const R* uy = ux + n3;
+        const R* uz = uy + n3;
+        // twice the components
+        const double wx = (widen(uz[sy]) - widen(uz[-sy])) - (widen(uy[sz]) - widen(uy[-sz]));
+        const double wy = (widen(ux[sz]) - widen(ux[-sz])) - (widen(uz[1]) - widen(uz[-1]));
+        const double wz = (widen(uy[1]) - widen(uy[-1])) - (widen(ux[sy]) - widen(ux[-sy]));
+        acc += quick_sqrt(fma(wx, wx, fma(wy, wy, wz * wz)));
     }
+    acc *= 0.5;
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     __shared__ double ws[kVortThreads / 32];
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
@@ -210,12 +253,14 @@ __global__ void __launch_bounds__(kVortThreads) k_vort_partial(const R* u, int E
     }
 }
 
-__global__ void k_vort_final(const double* partial, int nblocks, double count, double* out)
+// One block adds the block sums, each thread every 256th, in a fixed order.
+__global__ void __launch_bounds__(kVortThreads) k_vort_final(const double* partial, int nblocks, double count, double* out)
 {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    __shared__ double sh[kVortThreads / 32];
     double t = 0.0;
-    for (int b = 0; b < nblocks; b++) t += partial[b];
-    out[0] = t / count;
+    for (int b = threadIdx.x; b < nblocks; b += kVortThreads) t += partial[b];
+    t = block_sum(t, sh);
+    if (threadIdx.x == 0) out[0] = t / count;
 }
 
 cudaError_t launch_vorticity(const void* u, int u_f64, int E, int lo, int hi, double* scratch, double* out,
@@ -232,28 +277,35 @@ cudaError_t launch_vorticity(const void* u, int u_f64, int E, int lo, int hi, do
                                                                    scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_vort_final<<<1, 32, 0, s>>>(scratch, (int)g, (double)cube, out);
+    k_vort_final<<<1, kVortThreads, 0, s>>>(scratch, (int)g, (double)cube, out);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-__global__ void k_cons_final(const BoxDev* boxes, const ChainDev* chains, int nboxes, int64_t chunks,
-                             const double* partial, const double* vel, double* out, int32_t* status)
+// One block per box: the partials of its chunks and the momenta of its beads,
+// each thread every 256th of them (one thread for all of them took 108 us at
+// the 512 partials of a 128^3 box, a chain of dependent additions).
+__global__ void __launch_bounds__(kConsFinalThreads) k_cons_final(const BoxDev* boxes, const ChainDev* chains, int nboxes,
+                                                                  int64_t chunks, const double* partial,
+                                                                  const double* vel, double* out, int32_t* status)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nboxes) return;
+    const int b = blockIdx.x;
     const BoxDev& bd = boxes[b];
-    const int64_t nch = (bd.n3 + kConsChunk - 1) / kConsChunk;
+    const int64_t nch = min((bd.n3 + kConsChunk - 1) / kConsChunk, chunks);
     double t[4] = {0, 0, 0, 0};
-    for (int64_t c = 0; c < nch && c < chunks; c++)
+    for (int64_t c = threadIdx.x; c < nch; c += blockDim.x)
         for (int a = 0; a < 4; a++) t[a] += partial[((int64_t)b * chunks + c) * 4 + a];
     double pb[3] = {0, 0, 0};
     if (bd.chain >= 0) {
         const ChainDev& ch = chains[bd.chain];
-        for (int i = 0; i < ch.nbeads; i++)
+        for (int i = threadIdx.x; i < ch.nbeads; i += blockDim.x)
             for (int a = 0; a < 3; a++) pb[a] += vel[3 * (ch.bead_off + i) + a];
         for (int a = 0; a < 3; a++) pb[a] *= ch.mass;
     }
+    __shared__ double sh[kConsFinalThreads / 32];
+    for (int a = 0; a < 4; a++) t[a] = block_sum(t[a], sh);
+    for (int a = 0; a < 3; a++) pb[a] = block_sum(pb[a], sh);
+    if (threadIdx.x != 0) return;
     double* o = out + 8 * (int64_t)b;
     o[0] = (double)bd.n3 + t[0];
     for (int a = 0; a < 3; a++) {
