@@ -1389,43 +1389,46 @@ __global__ void k_init(typename Stor<ST>::E* Ab, BoxDev bd, const typename Stor<
 }
 
 // ---------------------------------------------------------------------------
-// Observables: density and velocity (what = 0: rho, 1: u) and raw deviations.
+// Observables: density and velocity (WHAT = 0: rho, 1: u) and raw deviations.
+//
+// A sweep over the populations that writes one or three reals per site: HBM
+// bound, the FP64 format by its arithmetic.  A thread takes VW consecutive
+// sites of a row and reads them with one vector load per population, all in
+// flight at once; the element the x shift needs from the neighbouring group
+// comes from the neighbouring lane (in FP64, whose time is arithmetic, from a
+// scalar load that hits the line the next lane fetches).  A site on an x face
+// reports its own stored values: one more predicated load per population puts
+// them in the place the shifted value would be taken from.  Rows on a y or z
+// face take the same loads without any shift.
+// Density / velocity read-out: 128^3 FP32 31 / 36 us (58 with a scalar load
+// per site and population; the bytes take 25 / 27), 256^3 binary16 115 / 151
+// (440; 104 / 123), 128^3 FP64 96 / 244 (293; 19 / 60 FP64 instructions a site,
+// of which the chip runs about 629 G a second).  Half as many sites a thread
+// measured 42 us and 150 - 224 us, scalar neighbours 34 / 43 and 133 / 177;
+// shuffles in FP64 140 / 302.
 // ---------------------------------------------------------------------------
-template <int ST>
-__global__ void k_fields(const typename Stor<ST>::E* Ab, BoxDev bd, int what, typename Stor<ST>::R* dst)
-{
-    using S = Stor<ST>;
-    using A = typename S::A;
-    const int Ei = bd.E, per = bd.per_mask;
-    const int64_t n3 = bd.n3;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n3; s += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(s % Ei), y = (int)((s / Ei) % Ei), z = (int)(s / ((int64_t)Ei * Ei));
-        const bool bnd = (!(per & 1) && (x == 0 || x == Ei - 1)) || (!(per & 2) && (y == 0 || y == Ei - 1)) ||
-                         (!(per & 4) && (z == 0 || z == Ei - 1));
-        A f[kQ], dr, j[3];
-        if (bnd) {
-            for (int i = 0; i < kQ; i++) f[i] = S::in(Ab[(int64_t)i * n3 + s]);
-        } else {
-            pull_site<ST>(Ab, n3, Ei, per, x, y, z, f);
-        }
-        moments<A>(f, dr, j);
-        const A rho = A(1) + dr;
-        if (what == 0) {
-            dst[s] = (typename S::R)rho;
-        } else {
-            for (int a = 0; a < 3; a++) {
-                const A ja = bnd ? j[a] : j[a] + A(0.5) * rho * (A)bd.accel[a];
-                dst[(int64_t)a * n3 + s] = (typename S::R)(ja / rho);
-            }
-        }
-    }
-}
+constexpr int kFieldsThreads = 256;
 
-template <int ST>
-__global__ void k_read_dev(const typename Stor<ST>::E* Ab, int64_t count, typename Stor<ST>::R* dst)
+// j / rho from r = 1 / rho, the product corrected by its own residual (within
+// one ulp), so that the three components share one reciprocal; the division
+// itself where the result is not finite.
+static __device__ __noinline__ double slow_ratio(double j, double rho) { return j / rho; }
+static __device__ __noinline__ float slow_ratio(float j, float rho) { return j / rho; }
+template <class A>
+__device__ __forceinline__ A ratio(A j, A rho, A r)
 {
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < count; s += (int64_t)gridDim.x * blockDim.x)
-        dst[s] = (typename Stor<ST>::R)Stor<ST>::in(Ab[s]);
+    const A q = j * r, t = fma(fma(-q, rho, j), r, q);
+    return isfinite(t) ? t : slow_ratio(j, rho);
+}
+// 1 / x: the hardware's approximation, in FP64 (about 20 bits) refined by two
+// Newton steps x' = x + x (1 - rho x).
+__device__ __forceinline__ float fast_inverse(float x) { return recip(x); }
+__device__ __forceinline__ double fast_inverse(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(fma(-x, y, 1.0), y, y);
+    return fma(fma(-x, y, 1.0), y, y);
 }
 
 // Density deviation and (WHAT = 1) momentum of one site from its populations,
@@ -1449,6 +1452,125 @@ __device__ __forceinline__ void site_moments(const F& f, A& r, A j[3])
             }
         }
     }
+}
+
+// The value of lane - 1 (up) or lane + 1.
+template <class E>
+__device__ __forceinline__ E shfl_elem(E v, bool up)
+{
+    return up ? __shfl_up_sync(0xffffffffu, v, 1) : __shfl_down_sync(0xffffffffu, v, 1);
+}
+template <>
+__device__ __forceinline__ uint16_t shfl_elem<uint16_t>(uint16_t v, bool up)
+{
+    const unsigned w = v;
+    return (uint16_t)(up ? __shfl_up_sync(0xffffffffu, w, 1) : __shfl_down_sync(0xffffffffu, w, 1));
+}
+
+template <int ST, int VW, int WHAT>
+__global__ void __launch_bounds__(kFieldsThreads) k_fields(const typename Stor<ST>::E* Ab, BoxDev bd,
+                                                            typename Stor<ST>::R* dst, int vec)
+{
+    using S = Stor<ST>;
+    using E = typename S::E;
+    using A = typename S::A;
+    using R = typename S::R;
+    using P = Pack<E, VW>;
+    using Raw = typename P::Raw;
+    constexpr bool kShuffle = sizeof(E) < 8;
+    const int Ei = bd.E, per = bd.per_mask, gpr = Ei / VW, fe = Ei * Ei;
+    const bool px = per & 1, py = per & 2, pz = per & 4;
+    const int n3 = (int)bd.n3, lane = threadIdx.x & 31;
+    for (int G = blockIdx.x * kFieldsThreads + threadIdx.x; G < n3 / VW; G += gridDim.x * kFieldsThreads) {
+        const int row = G / gpr, xg = G - row * gpr;
+        const int z = row / Ei, y = row - z * Ei;
+        const bool row_bnd = (!py && (y == 0 || y == Ei - 1)) || (!pz && (z == 0 || z == Ei - 1));
+        // offsets of the rows a population with c_y, c_z = +1 / -1 pulls from (none on a face row)
+        const int ym = row_bnd ? 0 : (y > 0 ? -Ei : fe - Ei), yp = row_bnd ? 0 : (y < Ei - 1 ? Ei : Ei - fe);
+        const int zm = row_bnd ? 0 : (z > 0 ? -fe : n3 - fe), zp = row_bnd ? 0 : (z < Ei - 1 ? fe : fe - n3);
+        const bool first = xg == 0, last = xg == gpr - 1;
+        const bool edge_l = !px && !row_bnd && first, edge_r = !px && !row_bnd && last;
+        const bool load_l = !kShuffle || first || lane == 0, load_r = !kShuffle || last || lane == 31;
+        const int nl = first ? Ei - 1 : -1, nr = last ? VW - Ei : VW;  // the neighbours' elements, from the group's first
+        P v[kQ];
+        E nb[kQ], own[kQ];
+        const E* pop = Ab + (int64_t)G * VW;
+#pragma unroll
+        for (int i = 0; i < kQ; i++, pop += n3) {
+            const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
+            const E* src = pop + ((cy > 0 ? ym : (cy < 0 ? yp : 0)) + (cz > 0 ? zm : (cz < 0 ? zp : 0)));
+            v[i].raw = ld_nc(reinterpret_cast<const Raw*>(src));
+            // an x-face site takes its own element in the neighbour's place ...
+            if (cx > 0 && load_l) nb[i] = __ldg(edge_l ? pop : src + nl);
+            if (cx < 0 && load_r) nb[i] = __ldg(edge_r ? pop + VW - 1 : src + nr);
+            // ... or in the place inside the group its shifted value comes from
+            if (cx > 0 || (cx == 0 && i > 0)) own[i] = edge_r ? __ldg(pop + VW - 1) : E(0);
+            if (cx < 0) own[i] = edge_l ? __ldg(pop) : E(0);
+            if (cx == 0 && i > 0 && edge_l) own[i] = __ldg(pop);
+        }
+        if constexpr (kShuffle) {  // n3 / VW is a multiple of 32: whole warps take part
+#pragma unroll
+            for (int i = 1; i < kQ; i++) {
+                const int cx = cvec(i, 0);
+                if (cx == 0) continue;
+                const E t = shfl_elem(v[i].e[cx > 0 ? VW - 1 : 0], cx > 0);
+                if (!(cx > 0 ? load_l : load_r)) nb[i] = t;
+            }
+        }
+#pragma unroll
+        for (int i = 1; i < kQ; i++) {
+            const int cx = cvec(i, 0);
+            if (cx > 0 && edge_r) v[i].e[VW - 2] = own[i];
+            if (cx < 0 && edge_l) v[i].e[1] = own[i];
+            if (cx == 0 && edge_l) v[i].e[0] = own[i];
+            if (cx == 0 && edge_r) v[i].e[VW - 1] = own[i];
+        }
+        __align__(16) R out[WHAT == 1 ? 3 : 1][VW];
+#pragma unroll
+        for (int k = 0; k < VW; k++) {
+            A r, j[3];
+            if (row_bnd)
+                site_moments<A, WHAT>([&](int i) { return S::in(v[i].e[k]); }, r, j);
+            else
+                site_moments<A, WHAT>(
+                    [&](int i) {
+                        const int cx = cvec(i, 0);
+                        if (cx > 0) return S::in(k == 0 ? nb[i] : v[i].e[k > 0 ? k - 1 : 0]);
+                        if (cx < 0) return S::in(k == VW - 1 ? nb[i] : v[i].e[k < VW - 1 ? k + 1 : k]);
+                        return S::in(v[i].e[k]);
+                    },
+                    r, j);
+            const A rho = A(1) + r;
+            if (WHAT == 0) {
+                out[0][k] = (R)rho;
+            } else {
+                if (bd.has_accel && !row_bnd && !(k == 0 && edge_l) && !(k == VW - 1 && edge_r))
+                    for (int a = 0; a < 3; a++) j[a] += A(0.5) * rho * (A)bd.accel[a];
+                const A inv = fast_inverse(rho);
+#pragma unroll
+                for (int a = 0; a < 3; a++) out[a][k] = (R)ratio(j[a], rho, inv);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < (WHAT == 1 ? 3 : 1); a++) {
+            R* o = dst + (int64_t)a * n3 + (int64_t)G * VW;
+            if (vec) {
+#pragma unroll
+                for (int q = 0; q < (int)(VW * sizeof(R) / 16); q++)
+                    reinterpret_cast<uint4*>(o)[q] = reinterpret_cast<const uint4*>(out[a])[q];
+            } else {
+#pragma unroll
+                for (int k = 0; k < VW; k++) o[k] = out[a][k];
+            }
+        }
+    }
+}
+
+template <int ST>
+__global__ void k_read_dev(const typename Stor<ST>::E* Ab, int64_t count, typename Stor<ST>::R* dst)
+{
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < count; s += (int64_t)gridDim.x * blockDim.x)
+        dst[s] = (typename Stor<ST>::R)Stor<ST>::in(Ab[s]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1714,13 +1836,30 @@ cudaError_t Launch<ST>::init(void* A, const BoxDev* boxes, int box, int64_t n3, 
     return cudaGetLastError();
 }
 
+template <int ST, int VW>
+cudaError_t launch_fields(const void* A, const BoxDev& bd, int what, void* dst, cudaStream_t s)
+{
+    using R = typename Stor<ST>::R;
+    const typename Stor<ST>::E* a = reinterpret_cast<const typename Stor<ST>::E*>(A);
+    const int grid = grid_for(bd.n3 / VW, kFieldsThreads, 1 << 20);
+    const int vec = reinterpret_cast<uintptr_t>(dst) % 16 == 0;  // the caller's buffer may start anywhere
+    if (what == 0)
+        k_fields<ST, VW, 0><<<grid, kFieldsThreads, 0, s>>>(a, bd, reinterpret_cast<R*>(dst), vec);
+    else
+        k_fields<ST, VW, 1><<<grid, kFieldsThreads, 0, s>>>(a, bd, reinterpret_cast<R*>(dst), vec);
+    return cudaGetLastError();
+}
+
 template <int ST>
 cudaError_t Launch<ST>::fields(const void* A, const BoxDev* boxes, int box, int64_t n3, int what, void* dst,
                                cudaStream_t s)
 {
-    k_fields<ST><<<grid_for(n3, 256), 256, 0, s>>>(reinterpret_cast<const typename Stor<ST>::E*>(A), boxes[box],
-                                                   what, reinterpret_cast<typename Stor<ST>::R*>(dst));
-    return cudaGetLastError();
+    // 16-byte loads; a row takes at least two groups (the two x faces lie in
+    // different ones), so 16-bit storage at E = 8 takes 8-byte loads
+        constexpr int VW = 16 / (int)sizeof(typename Stor<ST>::E);
+    if constexpr (VW == 8)
+        if (boxes[box].E < 2 * VW) return launch_fields<ST, VW / 2>(A, boxes[box], what, dst, s);
+    return launch_fields<ST, VW>(A, boxes[box], what, dst, s);
 }
 
 template <int ST>
