@@ -1492,6 +1492,21 @@ int32_t lb_mlp_forward(const void* params, int32_t K, const void* X, int64_t row
                        "lb_mlp_forward");
 }
 
+// The gradient and the loss go straight to device memory; anything else takes a copy behind the kernels.
+static cudaError_t train_rows(void* ws, int32_t K, int64_t batch_rows, const void* X, const float* T, int64_t rows,
+                              float* grad_out, double* loss_out, bool adam, float lr, int64_t t, cudaStream_t s)
+{
+    const MlpTrain W = mlp_train_layout(K, batch_rows);
+    const bool gd = grad_out && is_device_ptr(grad_out), ld = loss_out && is_device_ptr(loss_out);
+    const float* f = reinterpret_cast<const float*>(ws);
+    cudaError_t e = mlp_train(reinterpret_cast<unsigned char*>(ws), W, X, T, rows, gd ? grad_out : nullptr,
+                              ld ? loss_out : nullptr, adam, lr, t, s);
+    if (e == cudaSuccess && grad_out && !gd)
+        e = cudaMemcpyAsync(grad_out, f + W.grad, sizeof(float) * W.L.nmaster, cudaMemcpyDefault, s);
+    if (e == cudaSuccess && loss_out && !ld) e = cudaMemcpyAsync(loss_out, f + W.loss, sizeof(double), cudaMemcpyDefault, s);
+    return e;
+}
+
 int32_t lb_mlp_grad(void* ws, int32_t K, int64_t batch_rows, const void* X, const float* T, int64_t rows,
                     float* grad_out, double* loss_out, void* stream)
 {
@@ -1500,13 +1515,8 @@ int32_t lb_mlp_grad(void* ws, int32_t K, int64_t batch_rows, const void* X, cons
         g_last_error = "lb_mlp_grad: null pointer or rows outside [1, batch_rows]";
         return LB_ERR_ARG;
     }
-    const MlpTrain W = mlp_train_layout(K, batch_rows);
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    cudaError_t e = mlp_grad(reinterpret_cast<unsigned char*>(ws), W, X, T, rows, s);
-    float* f = reinterpret_cast<float*>(ws);
-    if (e == cudaSuccess && grad_out)
-        e = cudaMemcpyAsync(grad_out, f + W.grad, sizeof(float) * W.L.nmaster, cudaMemcpyDefault, s);
-    if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, f + W.loss, sizeof(double), cudaMemcpyDefault, s);
+    const cudaError_t e = train_rows(ws, K, batch_rows, X, T, rows, grad_out, loss_out, false, 0.f, 1,
+                                     reinterpret_cast<cudaStream_t>(stream));
     return cuda_status(e, "lb_mlp_grad");
 }
 
@@ -1518,12 +1528,8 @@ int32_t lb_mlp_train_step(void* ws, int32_t K, int64_t batch_rows, const void* X
         g_last_error = "lb_mlp_train_step: bad argument";
         return LB_ERR_ARG;
     }
-    const MlpTrain W = mlp_train_layout(K, batch_rows);
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    cudaError_t e = mlp_grad(reinterpret_cast<unsigned char*>(ws), W, X, T, rows, s);
-    if (e == cudaSuccess) e = mlp_adam(reinterpret_cast<unsigned char*>(ws), W, lr, t, s);
-    if (e == cudaSuccess && loss_out)
-        e = cudaMemcpyAsync(loss_out, reinterpret_cast<float*>(ws) + W.loss, sizeof(double), cudaMemcpyDefault, s);
+    const cudaError_t e = train_rows(ws, K, batch_rows, X, T, rows, nullptr, loss_out, true, lr, t,
+                                     reinterpret_cast<cudaStream_t>(stream));
     return cuda_status(e, "lb_mlp_train_step");
 }
 

@@ -4,9 +4,8 @@
 // boundary linearly between samples, Sec. 3; the residual network is an
 // added form).  Network: 24 features (padded to 32) -> 128 -> 128 -> 3K,
 // ReLU, BF16 weights and activations on the tensor cores with FP32
-// accumulation.  Training runs on the GPU: the forward and the backward on the
-// tcgen05 tensor cores (lbt_mlp_tc.cu), the loss and Adam on FP32 master
-// weights below.
+// accumulation.  This file: layouts, features and targets; forward on tcgen05
+// in lbt_mlp_tc.cu, training in lbt_mlp_train.cu.
 //
 // Layouts
 //   feature matrix X: bf16 [rows][32], row = (f E + q) E + p per box
@@ -151,64 +150,6 @@ __global__ void k_mlp_targets(const R* s_prev, const R* s0, const R* s1, const R
 }
 
 // ---------------------------------------------------------------------------
-// training: FP32 backward and Adam
-// ---------------------------------------------------------------------------
-// dY = 2 (Y - T) / (rows nout); loss += sum (Y - T)^2 / (rows nout)
-__global__ void k_mse(const float* Y, const float* T, int64_t n, float scale, float* dY, double* loss)
-{
-    double acc = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float d = Y[i] - T[i];
-        dY[i] = 2.f * d * scale;
-        acc += (double)d * d;
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc * scale);
-}
-
-// Adam on the master weights, then the bf16 / f32 inference copy.
-__global__ void k_adam(float* master, float* m, float* v, const float* grad, int64_t n, float lr, float b1, float b2,
-                       float eps, float c1, float c2)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float g = grad[i];
-        const float mi = b1 * m[i] + (1.f - b1) * g;
-        const float vi = b2 * v[i] + (1.f - b2) * g * g;
-        m[i] = mi;
-        v[i] = vi;
-        master[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    }
-}
-
-__global__ void k_export(const float* master, MlpLayout L, unsigned char* params)
-{
-    __nv_bfloat16* w1 = reinterpret_cast<__nv_bfloat16*>(params + L.w1);
-    __nv_bfloat16* w2 = reinterpret_cast<__nv_bfloat16*>(params + L.w2);
-    __nv_bfloat16* w3 = reinterpret_cast<__nv_bfloat16*>(params + L.w3);
-    float* b1 = reinterpret_cast<float*>(params + L.b1);
-    float* b2 = reinterpret_cast<float*>(params + L.b2);
-    float* b3 = reinterpret_cast<float*>(params + L.b3);
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    for (int e = tid; e < kMlpHidden * kMlpIn; e += nt) {  // W1t[o][i] = W1[i][o]
-        const int o = e / kMlpIn, i = e % kMlpIn;
-        w1[e] = __float2bfloat16_rn(master[L.m_w1 + i * kMlpHidden + o]);
-    }
-    for (int e = tid; e < kMlpHidden * kMlpHidden; e += nt) {
-        const int o = e / kMlpHidden, i = e % kMlpHidden;
-        w2[e] = __float2bfloat16_rn(master[L.m_w2 + i * kMlpHidden + o]);
-    }
-    for (int e = tid; e < L.nout * kMlpHidden; e += nt) {
-        const int o = e / kMlpHidden, i = e % kMlpHidden;
-        w3[e] = __float2bfloat16_rn(master[L.m_w3 + i * L.nout + o]);
-    }
-    for (int e = tid; e < kMlpHidden; e += nt) {
-        b1[e] = master[L.m_b1 + e];
-        b2[e] = master[L.m_b2 + e];
-    }
-    for (int e = tid; e < L.nout; e += nt) b3[e] = master[L.m_b3 + e];
-}
-
-// ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
 static int grid_cap(int64_t n, int threads)
@@ -280,51 +221,13 @@ MlpTrain mlp_train_layout(int K, int64_t B)
     W.m = take(P);
     W.v = take(P);
     W.grad = take(P);
-    W.h1 = take(B * kMlpHidden);
-    W.h2 = take(B * kMlpHidden);
-    W.y = take(B * W.L.nout);
-    W.dy = take(B * W.L.nout);
-    W.dh2 = take(B * kMlpHidden);
-    W.dh1 = take(B * kMlpHidden);
+    const int64_t tiles = (B + 127) / 128, parts = tiles < kMlpMaxPartials ? tiles : kMlpMaxPartials;
+    W.partial = take(parts * P);   // gradient of each block of the training kernel
+    W.loss_part = take(2 * parts);
     W.loss = take(2);  // one double
     W.params_byte = o * 4;
     W.bytes = al256(W.params_byte + W.L.bytes);
     return W;
-}
-
-cudaError_t mlp_grad(unsigned char* ws, const MlpTrain& W, const void* X, const float* T, int64_t rows, cudaStream_t s)
-{
-    float* f = reinterpret_cast<float*>(ws);
-    const MlpLayout& L = W.L;
-    const unsigned char* params = ws + W.params_byte;
-    // forward on tcgen05, saving the bf16 activations (h1, h2 hold bf16 rows)
-    cudaError_t e = mlp_forward_save_tc(X, rows, params, W.K, f + W.y, f + W.h1, f + W.h2, s);
-    if (e != cudaSuccess) return e;
-    cudaMemsetAsync(f + W.grad, 0, sizeof(float) * L.nmaster, s);
-    cudaMemsetAsync(f + W.loss, 0, sizeof(double), s);
-    const int64_t ny = rows * L.nout;
-    k_mse<<<grid_cap(ny, 256), 256, 0, s>>>(f + W.y, T, ny, 1.0f / (float)ny, f + W.dy,
-                                            reinterpret_cast<double*>(f + W.loss));
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // backward on tcgen05 (dh2, dh1 hold bf16 rows)
-    return mlp_backward_tc(X, rows, params, W.K, f + W.h1, f + W.h2, f + W.dy, f + W.dh2, f + W.dh1, f + W.grad, s);
-}
-
-cudaError_t mlp_adam(unsigned char* ws, const MlpTrain& W, float lr, int64_t t, cudaStream_t s)
-{
-    float* f = reinterpret_cast<float*>(ws);
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-    k_adam<<<grid_cap(W.L.nmaster, 256), 256, 0, s>>>(f + W.master, f + W.m, f + W.v, f + W.grad, W.L.nmaster, lr, b1,
-                                                       b2, eps, c1, c2);
-    return mlp_export(f + W.master, W.K, ws + W.params_byte, s);
-}
-
-cudaError_t mlp_export(const float* master, int K, void* params, cudaStream_t s)
-{
-    k_export<<<64, 256, 0, s>>>(master, mlp_layout(K), reinterpret_cast<unsigned char*>(params));
-    return cudaGetLastError();
 }
 
 __global__ void k_mlp_sets_from_ring(MlpFeatureSet* sets, int nsets, const BoxDev* boxes, const unsigned char* ring,

@@ -19,13 +19,16 @@ struct MlpLayout {
     int64_t m_w1, m_b1, m_w2, m_b2, m_w3, m_b3, nmaster;
 };
 
+// Blocks of the training kernel at most (its gradient partials in the workspace).
+constexpr int64_t kMlpMaxPartials = 160;
+
 // Float offsets of the training workspace (batch rows B), then the inference
 // parameters at params_byte.
 struct MlpTrain {
     MlpLayout L;
     int K;
     int64_t batch;
-    size_t master, m, v, grad, h1, h2, y, dy, dh2, dh1, loss;
+    size_t master, m, v, grad, partial, loss_part, loss;
     size_t params_byte, bytes;
 };
 
@@ -50,22 +53,16 @@ cudaError_t mlp_forward(const void* X, int64_t rows, const void* params, int K, 
 // residual at one substep is then read from consecutive rows).
 cudaError_t mlp_forward_tc(const void* X, int64_t rows, const void* params, int K, float* Y, int32_t* err,
                            cudaStream_t s, int64_t col_stride = 0);
-// Training forward on tcgen05: Y row-major [rows][3K] FP32 and the bf16
-// hidden activations after ReLU, H1 and H2 row-major [rows][128].
-cudaError_t mlp_forward_save_tc(const void* X, int64_t rows, const void* params, int K, float* Y, void* H1, void* H2,
-                                cudaStream_t s);
-// Backward on tcgen05 from dY (FP32 [rows][3K]): the FP32 gradient (master
-// layout, added to `grad`), with dH2 and dH1 (bf16 [rows][128]) as scratch.
-cudaError_t mlp_backward_tc(const void* X, int64_t rows, const void* params, int K, const void* H1, const void* H2,
-                            const float* dY, void* dH2, void* dH1, float* grad, cudaStream_t s);
+// Gradient and loss of rows (X, T) into the workspace (and to grad_out, loss_out
+// unless null: device memory), adam: followed by Adam step t with rate lr.
+cudaError_t mlp_train(unsigned char* ws, const MlpTrain& W, const void* X, const float* T, int64_t rows, float* grad_out,
+                      double* loss_out, bool adam, float lr, int64_t t, cudaStream_t s);
 cudaError_t mlp_features(const MlpFeatureSet* sets_dev, int nsets, int64_t total_rows, double u_max, int real_f64,
                          void* X, cudaStream_t s);
 // Features of one face set passed by value (6 E^2 rows from row 0).
 cudaError_t mlp_features_one(const MlpFeatureSet& set, double u_max, int real_f64, void* X, cudaStream_t s);
 cudaError_t mlp_targets(const void* const smp[4], const void* fine, int E, int K, int first_interval, double u_max,
                         int real_f64, float* T, cudaStream_t s);
-cudaError_t mlp_grad(unsigned char* ws, const MlpTrain& W, const void* X, const float* T, int64_t rows, cudaStream_t s);
-cudaError_t mlp_adam(unsigned char* ws, const MlpTrain& W, float lr, int64_t t, cudaStream_t s);
 cudaError_t mlp_export(const float* master, int K, void* params, cudaStream_t s);
 
 struct BoxDev;
