@@ -148,7 +148,7 @@ Layout plan_layout(const lb_box_desc* boxes, int nboxes, int storage, int ring_s
     L.step = off;
     off = align_up(off + sizeof(int64_t));
     L.tile_counter = off;
-    off = align_up(off + sizeof(int64_t));
+    off = align_up(off + 2 * sizeof(int64_t));
     L.faccel = off;  // frame-acceleration samples [box][ring slot][4]
     off = align_up(off + sizeof(double) * 4 * (size_t)nboxes * ring_slots);
     L.chain_accel = off;  // body acceleration of the step per chain [chain][4]
@@ -393,7 +393,7 @@ int enqueue_step(lb_ctx* ctx, int64_t n)
     sp.wait_ns = ctx->wait_ns;
     sp.withhold_tile = ctx->inject == LB_INJECT_WITHHOLD_LAST_TILE ? sp.total_tiles - 1 : -1;
     sp.hint_loads = nch > 0;
-    sp.pad_hint = 0;
+    sp.ends_step = nch == 0 && ctx->kernel == LB_KERNEL_STAGED;
     const bool timed = ctx->profiling && ctx->prof_used + 2 <= ctx->prof_ev.size();
     // inside a stream capture the timing events must become event-record nodes of the graph
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -411,6 +411,10 @@ int enqueue_step(lb_ctx* ctx, int64_t n)
     if (timed) {
         CK(cudaEventRecordWithFlags(ctx->prof_ev[ctx->prof_used + 1], ctx->stream, evflags));
         ctx->prof_used += 2;
+    }
+    if (sp.ends_step) {  // no forced sites, and the step has been advanced
+        ctx->a_is_pop_a = !ctx->a_is_pop_a;
+        return LB_OK;
     }
     if (nch > 0) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
     ForcedParams fp;

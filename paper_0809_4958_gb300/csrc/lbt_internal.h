@@ -154,13 +154,13 @@ struct SCParams {
     int32_t nboxes;
     int64_t total_tiles;
     const int64_t* step;          // device step counter n (state holds step n)
-    int64_t* tile_counter;        // next tile for the persistent staged kernel (zeroed every step)
+    int64_t* tile_counter;        // next tile for the persistent staged kernel, blocks out of tiles (both zeroed every step)
     int32_t* status;
     const FluctDev* fluct;        // [nboxes] fluctuating-collision parameters
     int64_t wait_ns;              // limit of the staged kernel's bounded barrier waits
     int64_t withhold_tile;        // test only: the staged producer never arms this tile (-1: none)
     int32_t hint_loads;           // 1: the staged bulk copies take the L2 evict-first policy (chains in the launch)
-    int32_t pad_hint;
+    int32_t ends_step;            // 1: no chain in the launch, the staged kernel advances the step and resets the counter
 };
 
 constexpr int64_t kWaitLimitNs = 1000000000;  // bounded device waits give up after one second
