@@ -393,6 +393,10 @@ int enqueue_step(lb_ctx* ctx, int64_t n)
     sp.wait_ns = ctx->wait_ns;
     sp.withhold_tile = ctx->inject == LB_INJECT_WITHHOLD_LAST_TILE ? sp.total_tiles - 1 : -1;
     sp.hint_loads = nch > 0;
+    // several boxes: runs of four neighbouring tiles where every SM takes more
+    // than 64, so that a producer meets a new box every fourth tile
+    sp.claim = ctx->nboxes > 1 && ctx->sms > 0 && sp.total_tiles > 64 * (int64_t)ctx->sms ? 4 : 1;
+    sp.pad_claim = 0;
     sp.ends_step = nch == 0 && ctx->kernel == LB_KERNEL_STAGED;
     const bool timed = ctx->profiling && ctx->prof_used + 2 <= ctx->prof_ev.size();
     // inside a stream capture the timing events must become event-record nodes of the graph

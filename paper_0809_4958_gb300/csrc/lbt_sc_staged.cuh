@@ -21,6 +21,8 @@
 // source lies outside are boundary sites, which are overwritten with the
 // boundary equilibrium anyway.
 #pragma once
+#include <cstddef>
+
 #include "lbt_device.cuh"
 #include "lbt_fluct.cuh"
 
@@ -44,7 +46,12 @@ struct Staged {
     static constexpr int kStageBytes = kQ * kRowStride;
     static constexpr int kFit = (227 * 1024 - kStagedHeaderBytes) / kStageBytes;
     static constexpr int kStages = kFit > kStagedMaxStages ? kStagedMaxStages : kFit;
-    static constexpr int kSmemBytes = kStagedHeaderBytes + kStages * kStageBytes;
+    // what is left of the shared memory holds the x-face boundary samples of
+    // each stage's rows (the paired bodies; see stage_edges)
+    static constexpr bool kEdges = SPT == 2 && ST != kF64;
+    static constexpr int kEdgeBytes =
+        kEdges ? (227 * 1024 - kStagedHeaderBytes - kStages * kStageBytes) / kStages / 16 * 16 : 0;
+    static constexpr int kSmemBytes = kStagedHeaderBytes + kStages * (kStageBytes + kEdgeBytes);
     static constexpr int kHalo = kStagedHaloBytes / (int)sizeof(E);         // halo elements
     static_assert(kStages >= 2, "tile too large for a two-stage pipeline");
     static_assert(kRowStride % 16 == 0, "bulk copies need 16-byte aligned rows");
@@ -186,6 +193,10 @@ struct StagedTile {
     int32_t slot[4];
     R c[4];
     A om, om1, srcfac, drho_b;  // 1/tau, 1 - 1/tau, 1 - 1/(2 tau), rho_b - 1
+    // x-face samples of the tile's rows in the stage (edge_stride 0: not
+    // staged): edge_n samples of weight edge_c, then the upsampler residual
+    int32_t edge_row, edge_stride, edge_n, edge_mlp;
+    R edge_c[4];
 };
 // Consumers keep reading a tile's header after they have released its data
 // stage (early release), so headers live in a ring of twice the stages: tile
@@ -456,6 +467,51 @@ struct PairIO<kBF16> {
     }
 };
 
+// Boundary velocity of the two adjacent sites x, x + 1 (x even) of a row on
+// face f (a y or z face, in-face row q): eight-byte loads, the arithmetic of
+// boundary_velocity and add_mlp_residual.
+template <int ST>
+__device__ __forceinline__ void boundary_velocity_pair(const SCParams& p, const StagedTile<ST>& th, int f, int q, int x,
+                                                       float2 u[3])
+{
+    const BoxDev& bd = th.bd;
+    const int64_t fe = (int64_t)bd.E * bd.E;
+    const float* ring = reinterpret_cast<const float*>(p.ring) + bd.ring_off + (3 * f) * fe + (int64_t)q * bd.E + x;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        u[c] = f2(0.f);
+#pragma unroll
+        for (int a = 0; a < 4; a++)
+            if (th.c[a] != 0.f)  // a zero weight never touches its (possibly unpushed) slot
+                u[c] = fma2(f2(th.c[a]), __ldg(reinterpret_cast<const float2*>(ring + (int64_t)th.slot[a] * p.ring_slot_elems + c * fe)),
+                            u[c]);
+    }
+    if (bd.mlp_row >= 0) {
+        const float* y = p.mlp_y + (int64_t)(3 * (th.mlp_s - 1)) * p.mlp_ystride + bd.mlp_row + f * fe + (int64_t)q * bd.E + x;
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+            u[c] = fma2(f2(p.mlp_yunit), __ldg(reinterpret_cast<const float2*>(y + c * p.mlp_ystride)), u[c]);
+    }
+}
+
+// Boundary velocity of a site on x face f (0 or 1) in box row `row` from the
+// samples staged with the tile.
+template <int ST>
+__device__ __forceinline__ void edge_velocity(const SCParams& p, const StagedTile<ST>& th, const float* edge, int f,
+                                              int row, float u[3])
+{
+    const int st = th.edge_stride;
+    const float* e = edge + 3 * f * st + (row - th.edge_row);
+#pragma unroll
+    for (int c = 0; c < 3; c++) u[c] = 0.f;
+    for (int a = 0; a < th.edge_n; a++, e += 6 * st)
+#pragma unroll
+        for (int c = 0; c < 3; c++) u[c] += th.edge_c[a] * e[c * st];
+    if (th.edge_mlp)
+#pragma unroll
+        for (int c = 0; c < 3; c++) u[c] += p.mlp_yunit * e[c * st];
+}
+
 // Consumer thread c (0 .. 479) of one tile of 960 sites takes the adjacent
 // sites s0 + 2c and s0 + 2c + 1 (same row: E and s0 are even), so a warp
 // reads and writes 64 consecutive sites with one word per lane.  Same
@@ -483,17 +539,13 @@ __device__ __forceinline__ void staged_tile_pair(const SCParams& p, const Staged
 
     const int s = s0 + 2 * tid;  // first site of the pair (even)
     const bool act = s < n3;     // n3 is even: both sites or none
-    int x, y, z;
-    {
-        const int sc = act ? s : 0;
-        const int row = div_e(sc, bd.div_magic);
-        x = sc - row * Ei;
-        z = div_e(row, bd.div_magic);
-        y = row - z * Ei;
-    }
-    const bool brow = (!py && (y == 0 || y == Ei - 1)) || (!pz && (z == 0 || z == Ei - 1));
-    const bool bnd0 = act && (brow || (!px && x == 0));
-    const bool bnd1 = act && (brow || (!px && x + 1 == Ei - 1));
+    const int row = div_e(act ? s : 0, bd.div_magic);
+    const int x = (act ? s : 0) - row * Ei;
+    const int z = div_e(row, bd.div_magic);
+    const int y = row - z * Ei;
+    const bool brow = act && ((!py && (y == 0 || y == Ei - 1)) || (!pz && (z == 0 || z == Ei - 1)));
+    const bool xface0 = act && !px && x == 0, xface1 = act && !px && x + 1 == Ei - 1;  // never both: E >= 8
+    const bool bnd0 = brow || xface0, bnd1 = brow || xface1;
     const bool keep0 = act && !bnd0, keep1 = act && !bnd1;
 
     // f_i pulled into both sites (zero where unused)
@@ -522,6 +574,11 @@ __device__ __forceinline__ void staged_tile_pair(const SCParams& p, const Staged
         // or zeroed elements only); it is multiplied by zero below
         f[i] = v;
     }
+    // x-face velocity: staged with the tile (read before the stage is released)
+    float ue[3];
+    const bool staged_edges = th.edge_stride != 0;
+    if ((xface0 || xface1) && staged_edges)
+        edge_velocity(p, th, reinterpret_cast<const float*>(stage + Staged<ST, 2>::kStageBytes), xface1, row, ue);
     __syncwarp();
     if ((tid & 31) == 0) mbar_arrive(empty);  // this warp is done with the stage
 
@@ -561,34 +618,38 @@ __device__ __forceinline__ void staged_tile_pair(const SCParams& p, const Staged
 
     // boundary sites: equilibrium of the boundary velocity from the ring
     if (bnd0 || bnd1) {
-        TimeWeights<float> tw;
-#pragma unroll
-        for (int a = 0; a < 4; a++) {
-            tw.slot[a] = th.slot[a];
-            tw.c[a] = th.c[a];
+        if (brow) {  // a row on a y or z face (its x-face sites, which belong to the x faces, follow)
+            const int f = !py && y == 0 ? 2 : (!py && y == Ei - 1 ? 3 : (z == 0 ? 4 : 5));
+            float2 u[3];
+            boundary_velocity_pair(p, th, f, f < 4 ? z : y, x, u);
+            ux = u[0];
+            uy = u[1];
+            uz = u[2];
+            drho = f2(th.drho_b);
         }
-        const float* ring = reinterpret_cast<const float*>(p.ring);
-#pragma unroll 1
-        for (int k = 0; k < 2; k++) {  // one lane at a time: fewer live registers
-            if (k == 0 ? bnd0 : bnd1) {
-                int pp, qq;
-                const int fc = owning_face(x + k, y, z, Ei, per, pp, qq);
-                float res[3];
-                load_mlp_residual(p, bd, th.mlp_s, fc, pp, qq, res);
-                float ub[3];
-                boundary_velocity<float>(ring, p.ring_slot_elems, bd, fc, pp, qq, tw, ub);
-                add_mlp_residual<float>(p, bd, res, ub);
-                if (k == 0) {
-                    drho.x = th.drho_b;
-                    ux.x = ub[0];
-                    uy.x = ub[1];
-                    uz.x = ub[2];
-                } else {
-                    drho.y = th.drho_b;
-                    ux.y = ub[0];
-                    uy.y = ub[1];
-                    uz.y = ub[2];
+        if (xface0 || xface1) {
+            if (!staged_edges) {
+                TimeWeights<float> tw;
+#pragma unroll
+                for (int a = 0; a < 4; a++) {
+                    tw.slot[a] = th.slot[a];
+                    tw.c[a] = th.c[a];
                 }
+                float res[3];
+                load_mlp_residual(p, bd, th.mlp_s, xface1, y, z, res);
+                boundary_velocity<float>(reinterpret_cast<const float*>(p.ring), p.ring_slot_elems, bd, xface1, y, z, tw, ue);
+                add_mlp_residual<float>(p, bd, res, ue);
+            }
+            if (xface0) {
+                drho.x = th.drho_b;
+                ux.x = ue[0];
+                uy.x = ue[1];
+                uz.x = ue[2];
+            } else {
+                drho.y = th.drho_b;
+                ux.y = ue[0];
+                uy.y = ue[1];
+                uz.y = ue[2];
             }
         }
         rho = add2(f2(1.f), drho);
@@ -799,7 +860,7 @@ __device__ __forceinline__ void staged_consume(const SCParams& p, unsigned char*
         if (b < 0) return;  // end of work
         const int64_t s0 = th.s0;
         const BoxDev& bd = th.bd;
-        const unsigned char* stage = smem + kStagedHeaderBytes + st * G::kStageBytes;
+        const unsigned char* stage = smem + kStagedHeaderBytes + st * (G::kStageBytes + G::kEdgeBytes);
         if (th.frozen) {
             // frozen box: release the stage, the state does not change
             __syncwarp();
@@ -838,15 +899,16 @@ __device__ __forceinline__ void staged_consume(const SCParams& p, unsigned char*
 
 // Prefetch into L2 (evict-last) of the upsampler residuals of substep ms for
 // the boundary sites of the box rows that tile [s0, s0 + T) covers: the
-// x-face sites at both ends of every row (faces 0 and 1, in-face (y, z)) and
-// whole rows on a y or z face, three components each.  One row per lane;
+// x-face sites at both ends of every row (faces 0 and 1, in-face (y, z);
+// staged: not those, they come with the tile) and whole rows on a y or z face,
+// three components each.  One row per lane;
 // every address lies inside the box's residual columns.
 __device__ __forceinline__ void prefetch_l2(const float* a)
 {
     asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(a));
 }
 __device__ __forceinline__ void prefetch_mlp_residuals(const SCParams& p, const BoxDev& bd, int ms, int64_t s0, int T,
-                                                       int lane)
+                                                       int lane, bool staged)
 {
     const int Eb = bd.E;
     const int64_t fe = (int64_t)Eb * Eb, str = p.mlp_ystride;
@@ -854,11 +916,12 @@ __device__ __forceinline__ void prefetch_mlp_residuals(const SCParams& p, const 
     const int64_t r_first = s0 / Eb, r_end = (s0 + T - 1) / Eb + 1;
     for (int64_t r = r_first + lane; r < r_end && r < fe; r += 32) {
         const int yy = (int)(r % Eb), zz = (int)(r / Eb);
+        if (!staged)
 #pragma unroll
-        for (int c = 0; c < 3; c++) {
-            prefetch_l2(y0 + c * str + (int64_t)zz * Eb + yy);       // x- face
-            prefetch_l2(y0 + c * str + fe + (int64_t)zz * Eb + yy);  // x+ face
-        }
+            for (int c = 0; c < 3; c++) {
+                prefetch_l2(y0 + c * str + (int64_t)zz * Eb + yy);       // x- face
+                prefetch_l2(y0 + c * str + fe + (int64_t)zz * Eb + yy);  // x+ face
+            }
         const int fo = yy == 0 ? 2 : (yy == Eb - 1 ? 3 : (zz == 0 ? 4 : (zz == Eb - 1 ? 5 : -1)));
         if (fo >= 0) {
             const int q = fo < 4 ? zz : yy;  // in-face (x, z) on a y face, (x, y) on a z face
@@ -870,15 +933,70 @@ __device__ __forceinline__ void prefetch_mlp_residuals(const SCParams& p, const 
     }
 }
 
+// The samples of the x faces (sites x = 0 and E - 1) of the box rows a tile
+// covers.  In a face sample [3][z][y] row (y, z) of the box is element z E + y,
+// so the tile's rows are one run per face, component and sample: one bulk copy
+// each, next to the tile's populations, in place of the loads from global
+// memory that every warp with the end of a row waited for.  Lane k takes
+// sample k / 6 of those with a weight, then the upsampler's residuals of the
+// substep; face (k % 6) / 3, component k % 3.  Runs are `stride` elements long,
+// start at a multiple of four (16 bytes) and lie inside E^2, itself a multiple
+// of 64.  Boxes whose runs do not fit the room of a stage (short rows, many
+// samples) load from global memory.  Fills the header's fields; returns the
+// run's base (null: none), E^2 - stride in last_start.  (With the producer's
+// work per box: 128 boxes of 64^3 with the upsampler 1198 -> 846 us a step, 512
+// uneven boxes with chains 1817 -> 1496.)
+template <int ROOM, int ST>
+__device__ __forceinline__ const float* edge_runs(const SCParams& p, StagedTile<ST>& th, int T, int lane, int& last_start)
+{
+    const BoxDev& bd = th.bd;
+    const int fe = bd.E * bd.E;
+    const int stride = ((T + bd.E - 2) / bd.E + 1 + 3 + 3) & ~3;  // rows a tile may touch, from a multiple of four
+    int ns = 0, my_slot = 0;
+    float my_c = 0.f;
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+        if (th.c[a] != 0.f) {  // a zero weight never touches its (possibly unpushed) slot
+            if (lane / 6 == ns) my_slot = th.slot[a];
+            if (lane == ns) my_c = th.c[a];
+            ns++;
+        }
+    const bool mlp = bd.mlp_row >= 0;
+    const int runs = 6 * (ns + (mlp ? 1 : 0));
+    const bool fits = !(bd.per_mask & 1) && !bd.fluct && runs <= 32 && runs * stride * 4 <= ROOM && stride <= fe;
+    if (lane < 4) th.edge_c[lane] = my_c;
+    if (lane == 0) {
+        th.edge_stride = fits ? stride : 0;
+        th.edge_n = ns;
+        th.edge_mlp = mlp;
+    }
+    last_start = fe - stride;
+    if (!fits || lane >= runs) return nullptr;
+    const int k = lane % 6;
+    return lane < 6 * ns ? reinterpret_cast<const float*>(p.ring) + (int64_t)my_slot * p.ring_slot_elems + bd.ring_off +
+                               (int64_t)k * fe
+                         : p.mlp_y + (int64_t)(3 * (th.mlp_s - 1) + k % 3) * p.mlp_ystride + bd.mlp_row + (int64_t)(k / 3) * fe;
+}
+
 // Producer warp (the last warp): claims tiles from the global counter (reset
-// to zero by the forced re-collision at the end of every step, so a block that
-// starts late -- its SM still busy with the bead kernel -- simply takes fewer
-// tiles) and fills the stages as the consumers free them.  Lane 0 claims,
-// waits for the stage and writes the tile header; lane i < 19 handles
-// population row i: its source range, the zeroing of the part of the row that
-// lies outside the box's arrays (those sites are boundary sites: their pulled
-// values are multiplied by zero and must be finite, so no consumer may read
-// what a previous tile left there), and its bulk copy.
+// to zero at the end of every step, so a block that starts late -- its SM
+// still busy with the bead kernel -- simply takes fewer tiles) and fills the
+// stages as the consumers free them.  Lane 0 claims and waits for the stage;
+// lane i < 19 handles population row i: its source range, the zeroing of the
+// part of the row that lies outside the box's arrays (those sites are boundary
+// sites: their pulled values are multiplied by zero and must be finite, so no
+// consumer may read what a previous tile left there), and its bulk copy.
+//
+// One tile's pass through this loop must stay below what the consumers take
+// for a tile (2.2 us at 256^3 in 16-bit storage), or the copies starve.  The
+// header and everything that depends on the box alone is therefore worked out
+// when the box changes (records, status and samples from global memory, a few
+// round trips) and kept in registers, the header as words spread over the
+// lanes; a further tile of the box only stores them.  Launches with many tiles
+// to a block claim several neighbours at once for the same reason.  (Worked out
+// for every tile, 256^3 binary16 took 268 us a step and takes 220, 128^3 FP32
+// under a body force 71.6 and 58.7; one more round trip a tile made them 330
+// and 83.)
 template <int ST, int SPT, int KIND>
 __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char* smem, StagedHeader<ST>* hd, int64_t n)
 {
@@ -886,7 +1004,11 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
     using E = typename Stor<ST>::E;
     using R = typename Stor<ST>::R;
     using A = typename Stor<ST>::A;
+    using Tile = StagedTile<ST>;
     constexpr int T = G::kSites, H = G::kHalo, W = T + 2 * H;
+    constexpr int kWords = (int)(sizeof(Tile) / 8), kMine = (kWords + 31) / 32;  // header words, of one lane
+    static_assert(sizeof(Tile) % 8 == 0 && offsetof(Tile, s0) % 8 == 0 && offsetof(Tile, bd) == 0, "header copied by words");
+    static_assert(sizeof(BoxDev) % 8 == 0 && sizeof(BoxDev) / 8 <= 32, "box record copied by one warp");
     const int lane = threadIdx.x & 31;
     int cy = 0, cz = 0;  // y and z components of this lane's population
 #pragma unroll
@@ -897,14 +1019,28 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
         }
     const uint64_t pol = p.hint_loads ? l2_evict_first_policy() : 0;
     unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p.tile_counter);
-    long long next = lane == 0 ? (long long)atomicAdd(ctr, 1ull) : 0;
-    next = __shfl_sync(0xffffffffu, next, 0);
+    const int run = p.claim;  // neighbouring tiles of one claim
     const bool back = (n & 1) && p.withhold_tile < 0;
-    int last_b = -1;
-    TimeWeights<R> tw{};
-    int mlp_s = 0;
+    long long next = lane == 0 ? (long long)atomicAdd(ctr, (unsigned long long)run) : 0;
+    next = __shfl_sync(0xffffffffu, next, 0);
+    int left = run;  // tiles of the claim not yet taken
+    // of the current box
+    int64_t tile_lo = 0, tile_hi = 0;  // its tiles
+    uint64_t hw[kMine];
+    const E* row_src = nullptr;        // this lane's population, at its pull shift
+    int64_t n3 = 0;
+    int Ei = 1, fe = 1, shift = 0;
+    uint64_t div_magic = 0;
+    const float* edge_src = nullptr;
+    int edge_bytes = 0, edge_last = 0, ms = 0;
+    bool mlp = false;
     for (int k = 0;; k++) {
         const int st = k % G::kStages;
+        // odd steps sweep the tiles backwards: what the last step wrote last is
+        // read first, out of L2 where it still lies (128^3 FP32 with a chain
+        // 63.2 -> 61.6 us a step; larger boxes lose nothing)
+        const int64_t t = back && next < p.total_tiles ? p.total_tiles - 1 - next : next;
+        Tile& th = hd->t[k % (2 * G::kStages)];
         // the stage's previous tile must be released by all consumer warps; if
         // that does not happen within the limit the consumers have left
         if (k >= G::kStages) {
@@ -912,65 +1048,92 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
             if (lane == 0) ok = mbar_wait_bounded(&hd->empty[st], (uint32_t)(((k / G::kStages) - 1) & 1), p.wait_ns);
             if (!__shfl_sync(0xffffffffu, ok, 0)) return;
         }
-        // odd steps sweep the tiles backwards: what the last step wrote last is
-        // read first, out of L2 where it still lies (128^3 FP32 with a chain
-        // 63.2 -> 61.6 us a step; larger boxes lose nothing)
-        const int64_t t = back && next < p.total_tiles ? p.total_tiles - 1 - next : next;
-        StagedTile<ST>& th = hd->t[k % (2 * G::kStages)];
         if (t >= p.total_tiles) {
             if (lane == 0) {
                 th.box = -1;
                 mbar_arrive(&hd->full[st]);  // completes the phase with no bytes: end of work
             }
-            // no tile left for this block: the kernel after this one (the
-            // forced re-collision, a programmatic dependent) may be scheduled
-            // once every block has got here; it waits on the device for this
-            // grid to complete
+            // no tile left for this block: the kernel after this one (a
+            // programmatic dependent) may be scheduled once every block has
+            // got here; it waits on the device for this grid to complete
             asm volatile("griddepcontrol.launch_dependents;");
             return;
         }
-        if (lane == 0) next = (long long)atomicAdd(ctr, 1ull);  // the next claim overlaps this tile's copies
-        const int b = locate_box_warp(p, t, lane);
-        const BoxDev& bd = p.boxes[b];
-        const int64_t s0 = (t - p.tile_prefix[b]) * T;
-        // header: the box record word by word across the lanes, the rest by lane 0
-        static_assert(sizeof(BoxDev) % 8 == 0 && sizeof(BoxDev) / 8 <= 32, "box record copied by one warp");
-        if (lane < (int)(sizeof(BoxDev) / 8))
-            reinterpret_cast<uint64_t*>(&th.bd)[lane] = reinterpret_cast<const uint64_t*>(&bd)[lane];
-        __syncwarp();
-        if (lane == 0) {
-            if (b != last_b) {  // boundary-layer constants of this box at step n
-                tw = time_weights<R>(n, bd.K, bd.time_interp, p.ring_slots);
-                mlp_s = bd.mlp_row >= 0 ? mlp_substep(n, bd.K) : 0;
-                last_b = b;
+        long long claimed = 0;
+        if (left == 1 && lane == 0) claimed = (long long)atomicAdd(ctr, (unsigned long long)run);  // overlaps this tile's copies
+        if (t < tile_lo || t >= tile_hi) {  // another box: its record and what the collision and the boundary need at this step
+            const int b = locate_box_warp(p, t, lane);
+            const BoxDev& bd = p.boxes[b];
+            tile_lo = p.tile_prefix[b];
+            tile_hi = p.tile_prefix[b + 1];
+            if (lane < (int)(sizeof(BoxDev) / 8))
+                reinterpret_cast<uint64_t*>(&th.bd)[lane] = reinterpret_cast<const uint64_t*>(&bd)[lane];
+            const int frozen = p.status[b] != 0;
+            __syncwarp();
+            if (lane == 0) {
+                const TimeWeights<R> tw = time_weights<R>(n, th.bd.K, th.bd.time_interp, p.ring_slots);
+                th.mlp_s = th.bd.mlp_row >= 0 ? mlp_substep(n, th.bd.K) : 0;
+                if (KIND > 0 && th.bd.frame) {  // the header carries the body acceleration of step n (frame
+                                                // boxes carry a body force, so they run a general kernel)
+                    double a[3];
+                    frame_accel_at(th.bd, p.faccel, p.ring_slots, n, a);
+                    for (int c = 0; c < 3; c++) th.bd.accel[c] = a[c];
+                }
+                th.box = b;
+                th.frozen = frozen;
+                for (int a = 0; a < 4; a++) {
+                    th.slot[a] = tw.slot[a];
+                    th.c[a] = tw.c[a];
+                }
+                th.om = A(1) / (A)th.bd.tau;
+                th.om1 = A(1) - th.om;
+                th.srcfac = A(1) - A(0.5) * th.om;
+                th.drho_b = (A)th.bd.rho_b - A(1);
             }
-            if (KIND > 0 && bd.frame) {  // the header carries the body acceleration of step n (frame
-                                         // boxes carry a body force, so they run a general kernel)
-                double a[3];
-                frame_accel_at(bd, p.faccel, p.ring_slots, n, a);
-                for (int c = 0; c < 3; c++) th.bd.accel[c] = a[c];
+            __syncwarp();
+            Ei = th.bd.E;
+            fe = Ei * Ei;
+            n3 = th.bd.n3;
+            div_magic = th.bd.div_magic;
+            shift = cy * Ei + cz * fe + H;
+            row_src = reinterpret_cast<const E*>(p.A) + th.bd.f_off + (int64_t)(lane < kQ ? lane : 0) * n3;
+            ms = th.mlp_s;
+            mlp = th.bd.mlp_row >= 0 && ms > 0;
+            if constexpr (G::kEdges) {
+                edge_src = edge_runs<G::kEdgeBytes>(p, th, T, lane, edge_last);
+                __syncwarp();
+                edge_bytes = edge_src ? th.edge_stride * 4 : 0;
             }
-            th.box = b;
-            th.s0 = s0;
-            th.mlp_s = mlp_s;
-            th.frozen = p.status[b] != 0;
-            for (int a = 0; a < 4; a++) {
-                th.slot[a] = tw.slot[a];
-                th.c[a] = tw.c[a];
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < kMine; q++)
+                if (lane + 32 * q < kWords) hw[q] = reinterpret_cast<const uint64_t*>(&th)[lane + 32 * q];
+            __syncwarp();
+        }
+        const int64_t s0 = (t - tile_lo) * T;
+        int edge_first = 0;
+        if constexpr (G::kEdges) edge_first = min(div_e(s0, div_magic) & ~3, edge_last);
+        // the header, with this tile's own words
+#pragma unroll
+        for (int q = 0; q < kMine; q++) {
+            const int w = lane + 32 * q;
+            if (w < kWords) {
+                uint64_t v = hw[q];
+                if (w == (int)(offsetof(Tile, s0) / 8)) v = (uint64_t)s0;
+                if (w == (int)(offsetof(Tile, edge_row) / 8)) {
+                    const uint64_t r = (uint32_t)edge_first;
+                    v = offsetof(Tile, edge_row) % 8 ? (v & 0xffffffffull) | (r << 32) : (v & ~0xffffffffull) | r;
+                }
+                reinterpret_cast<uint64_t*>(&th)[w] = v;
             }
-            th.om = A(1) / (A)bd.tau;
-            th.om1 = A(1) - th.om;
-            th.srcfac = A(1) - A(0.5) * th.om;
-            th.drho_b = (A)bd.rho_b - A(1);
         }
         // row `lane`: source range clamped to the box's arrays
-        unsigned char* stage = smem + kStagedHeaderBytes + st * G::kStageBytes;
-        const int64_t Ei = bd.E, n3 = bd.n3;
-        const int64_t start = s0 - (cy * Ei + cz * Ei * Ei) - H;
+        unsigned char* stage = smem + kStagedHeaderBytes + st * (G::kStageBytes + G::kEdgeBytes);
+        const int64_t start = s0 - shift;
         const int64_t lo = start > 0 ? start : 0;
         const int64_t hi = start + W < n3 ? start + W : n3;
         const bool mine = lane < kQ && hi > lo;
-        uint32_t bytes = mine ? (uint32_t)((hi - lo) * sizeof(E)) : 0u;
+        const uint32_t bytes = mine ? (uint32_t)((hi - lo) * sizeof(E)) : 0u;
         if (lane < kQ) {
             const int a = mine ? (int)(lo - start) : W;  // first copied element
             const int e = mine ? (int)(hi - start) : W;  // end of the copied elements
@@ -981,35 +1144,35 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
                 for (int x = e; x < W; x += per16) row[x / per16] = make_uint4(0, 0, 0, 0);
             }
         }
-        uint32_t total = bytes;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-        next = __shfl_sync(0xffffffffu, next, 0);
+        const uint32_t total = __reduce_add_sync(0xffffffffu, bytes + (uint32_t)edge_bytes);
         __syncwarp();  // header and zeroed parts written before the stage is armed
         if (t == p.withhold_tile) {
             // test only: this stage is never armed and no copy is issued, so
             // its full barrier never completes and the consumers' bounded wait
             // runs out (the header above is in place for them to name the box)
             __threadfence_block();
-            continue;
+        } else {
+            if (lane == 0) mbar_arrive_expect_tx(&hd->full[st], total);
+            __syncwarp();
+            if (mine) {
+                fence_proxy_async_smem();
+                unsigned char* dst = stage + lane * G::kRowStride + (lo - start) * sizeof(E);
+                if (p.hint_loads) bulk_load_hint(dst, row_src + lo, bytes, &hd->full[st], pol);
+                else bulk_load(dst, row_src + lo, bytes, &hd->full[st]);
+            }
+            if (edge_bytes)
+                bulk_load(stage + G::kStageBytes + lane * edge_bytes, edge_src + edge_first, (uint32_t)edge_bytes, &hd->full[st]);
+            // upsampler boxes: the residuals the tile's boundary sites will add
+            // come from an output far larger than L2; prefetch them into L2 while
+            // the copies are in flight, so that the consumers' loads hit there
+            if (mlp) prefetch_mlp_residuals(p, th.bd, ms, s0, T, lane, th.edge_stride != 0);
         }
-        if (lane == 0) mbar_arrive_expect_tx(&hd->full[st], total);
-        __syncwarp();
-        if (mine) {
-            fence_proxy_async_smem();
-            const E* Ab = reinterpret_cast<const E*>(p.A) + bd.f_off;
-            if (p.hint_loads)
-                bulk_load_hint(stage + lane * G::kRowStride + (lo - start) * sizeof(E), Ab + (int64_t)lane * n3 + lo,
-                               bytes, &hd->full[st], pol);
-            else
-                bulk_load(stage + lane * G::kRowStride + (lo - start) * sizeof(E), Ab + (int64_t)lane * n3 + lo, bytes,
-                          &hd->full[st]);
+        if (--left > 0) {
+            next++;
+        } else {
+            next = __shfl_sync(0xffffffffu, claimed, 0);
+            left = run;
         }
-        // upsampler boxes: the residuals the tile's boundary sites will add
-        // come from an output far larger than L2; prefetch them into L2 while
-        // the copies are in flight, so that the consumers' loads hit there
-        const int ms = __shfl_sync(0xffffffffu, mlp_s, 0);
-        if (bd.mlp_row >= 0 && ms > 0) prefetch_mlp_residuals(p, bd, ms, s0, T, lane);
     }
 }
 
