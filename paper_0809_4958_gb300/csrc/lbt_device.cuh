@@ -158,6 +158,24 @@ __device__ __forceinline__ float unit_uniform_t<float>(uint32_t v)
     return 1.7320508075688772f * (2.0f * u01 - 1.0f);
 }
 
+// 1 / x by the hardware's approximation: in FP32 PTX rcp.approx.ftz.f32 (at
+// most one ulp), in FP64 about 20 bits refined by one third-order step
+// x' = x (1 + e + e^2), e = 1 - a x, which leaves e^3; without the branch of the
+// library's division, so that independent reciprocals interleave (an FP64
+// instruction takes some 64 cycles to its result).
+__device__ __forceinline__ double fast_inverse(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float fast_inverse(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 // Reciprocal of the bead pair forces: correctly rounded division in FP64,
 // the hardware's approximate reciprocal in FP32 (PTX rcp.approx.ftz.f32, at
 // most one ulp off, far below the FP32 dynamics' own rounding; the pair
@@ -171,6 +189,11 @@ __device__ __forceinline__ float recip(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+
+// 1 / rho of a collided site: in FP64 by fast_inverse (the FP64 pipe bounds
+// that collision), the division in FP32.
+__device__ __forceinline__ double site_inverse(double rho) { return fast_inverse(rho); }
+__device__ __forceinline__ float site_inverse(float rho) { return 1.0f / rho; }
 
 __device__ __forceinline__ int wrapi(int v, int E) { return v < 0 ? v + E : (v >= E ? v - E : v); }
 

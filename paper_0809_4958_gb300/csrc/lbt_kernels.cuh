@@ -1420,17 +1420,6 @@ __device__ __forceinline__ A ratio(A j, A rho, A r)
     const A q = j * r, t = fma(fma(-q, rho, j), r, q);
     return isfinite(t) ? t : slow_ratio(j, rho);
 }
-// 1 / x: the hardware's approximation, in FP64 (about 20 bits) refined by two
-// Newton steps x' = x + x (1 - rho x).
-__device__ __forceinline__ float fast_inverse(float x) { return recip(x); }
-__device__ __forceinline__ double fast_inverse(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(fma(-x, y, 1.0), y, y);
-    return fma(fma(-x, y, 1.0), y, y);
-}
-
 // Density deviation and (WHAT = 1) momentum of one site from its populations,
 // by opposite pairs: their sums make the density, their differences the
 // momentum (39 additions in place of 48).

@@ -193,6 +193,7 @@ struct StagedTile {
     int32_t slot[4];
     R c[4];
     A om, om1, srcfac, drho_b;  // 1/tau, 1 - 1/tau, 1 - 1/(2 tau), rho_b - 1
+    A acc[3], pad;              // body acceleration of the step
     // x-face samples of the tile's rows in the stage (edge_stride 0: not
     // staged): edge_n samples of weight edge_c, then the upsampler residual
     int32_t edge_row, edge_stride, edge_n, edge_mlp;
@@ -216,12 +217,16 @@ static_assert(sizeof(StagedHeader<kF32>) <= kStagedHeaderBytes, "header does not
 // q = (s * m) >> 40 with m = ceil(2^40 / E), exact for s < 2^31 and E <= 1024.
 __device__ __forceinline__ int div_e(int64_t s, uint64_t m) { return (int)(((uint64_t)s * m) >> 40); }
 
-// Consumer thread c (0 .. 479) of one tile: sites s0 + c + k 480, so the lanes
-// of a warp read consecutive shared-memory words and store consecutive global
-// words.  Populations go to registers, the warp releases the stage, then the
-// collision (BGK with the equilibrium of opposite pairs shared: the even part
-// in c.u is common, the odd part changes sign) and the stores.
-template <int ST, int SPT, bool PER, bool ACCEL>
+// One site per consumer thread (FP64, and the reduced formats with one site a
+// thread): thread c (0 .. 479) takes site s0 + c, so the lanes of a warp read
+// consecutive shared-memory words and store consecutive global words.  The
+// site's populations go to registers, the warp releases the stage, then the
+// collision (BGK by opposite pairs, whose equilibrium has an even part in
+// common and an odd part that changes sign) and the stores.  FP64 is bound by
+// its arithmetic (two lanes a clock on an SM), so its instructions are counted:
+// about 125 a site in place of 212 (each population's momentum and relaxation
+// by itself, a division), 128^3 in 544 us in place of 713.
+template <int ST, bool PER, bool ACCEL>
 __device__ __forceinline__ void staged_tile(const SCParams& p, const StagedTile<ST>& th, const unsigned char* stage,
                                             uint64_t* empty)
 {
@@ -229,182 +234,137 @@ __device__ __forceinline__ void staged_tile(const SCParams& p, const StagedTile<
     using E = typename S::E;
     using A = typename S::A;
     using R = typename S::R;
-    constexpr int H = Staged<ST, SPT>::kHalo;
-    constexpr int C = kStagedConsumers;
+    constexpr int H = Staged<ST, 1>::kHalo;
     const int tid = threadIdx.x;
     // site indices of a box fit 32 bits (E <= 1024)
-    const int s0 = (int)th.s0;
+    const int s = (int)th.s0 + tid;
     const BoxDev& bd = th.bd;
-
     const int Ei = bd.E;
     const int n3 = (int)bd.n3;
-    // body acceleration of the step in the arithmetic type, converted once
-    A acA[3] = {A(0), A(0), A(0)};
-    if (ACCEL)
-        for (int c = 0; c < 3; c++) acA[c] = (A)bd.accel[c];
-    const uint64_t mE = bd.div_magic;
     const int per = bd.per_mask;
     const bool px = per & 1, py = per & 2, pz = per & 4;
     const E* Ab = reinterpret_cast<const E*>(p.A) + bd.f_off;
     E* Bb = reinterpret_cast<E*>(p.B) + bd.f_off;
 
-    // coordinates of site k (recomputed where needed rather than held in
-    // registers across the population loads)
-    auto coords = [&](int k, int& x, int& y, int& z) {
-        const int s = s0 + tid + k * C;
-        const int sc = s < n3 ? s : 0;
-        const int row = div_e(sc, mE);
-        x = sc - row * Ei;
-        z = div_e(row, mE);
-        y = row - z * Ei;
-    };
-    int xs_[SPT], ys_[SPT], zs_[SPT];
-    bool act[SPT], bnd[SPT];
-    bool any_bnd = false;
-#pragma unroll
-    for (int k = 0; k < SPT; k++) {
-        act[k] = s0 + tid + k * C < n3;
-        int x, y, z;
-        coords(k, x, y, z);
-        xs_[k] = x;
-        ys_[k] = y;
-        zs_[k] = z;
-        bnd[k] = act[k] && ((!px && (x == 0 || x == Ei - 1)) || (!py && (y == 0 || y == Ei - 1)) ||
-                            (!pz && (z == 0 || z == Ei - 1)));
-        any_bnd |= bnd[k];
-    }
+    const bool act = s < n3;
+    const int row = div_e(act ? s : 0, bd.div_magic);
+    const int x = (act ? s : 0) - row * Ei;
+    const int z = div_e(row, bd.div_magic);
+    const int y = row - z * Ei;
+    const bool bnd = act && ((!px && (x == 0 || x == Ei - 1)) || (!py && (y == 0 || y == Ei - 1)) ||
+                             (!pz && (z == 0 || z == Ei - 1)));
 
-    // f_i pulled into site k: shared memory, or global memory across a periodic
-    // wrap; zero where it is not used (boundary and inactive sites)
-    A f[kQ][SPT];
+    // f_i pulled into the site: shared memory, or global memory across a
+    // periodic wrap; zero where it is not used (boundary and inactive sites)
+    A f[kQ];
 #pragma unroll
     for (int i = 0; i < kQ; i++) {
         const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
-        const E* row = reinterpret_cast<const E*>(stage + i * Staged<ST, SPT>::kRowStride);
-#pragma unroll
-        for (int k = 0; k < SPT; k++) {
-            A v = S::in(row[H + tid + k * C - cx]);
-            if (PER) {
-                const int xs = xs_[k] - cx, ys = ys_[k] - cy, zs = zs_[k] - cz;
-                const bool wrap = (px && (xs < 0 || xs >= Ei)) || (py && (ys < 0 || ys >= Ei)) ||
-                                  (pz && (zs < 0 || zs >= Ei));
-                if (wrap && act[k])
-                    v = S::in(Ab[(int64_t)i * n3 + ((int64_t)wrapi(zs, Ei) * Ei + wrapi(ys, Ei)) * Ei + wrapi(xs, Ei)]);
-            }
-            f[i][k] = (act[k] && !bnd[k]) ? v : A(0);
+        A v = S::in(reinterpret_cast<const E*>(stage + i * Staged<ST, 1>::kRowStride)[H + tid - cx]);
+        if (PER) {
+            const int xs = x - cx, ys = y - cy, zs = z - cz;
+            const bool wrap = (px && (xs < 0 || xs >= Ei)) || (py && (ys < 0 || ys >= Ei)) ||
+                              (pz && (zs < 0 || zs >= Ei));
+            if (wrap && act)
+                v = S::in(Ab[(int64_t)i * n3 + ((int64_t)wrapi(zs, Ei) * Ei + wrapi(ys, Ei)) * Ei + wrapi(xs, Ei)]);
         }
+        f[i] = act && !bnd ? v : A(0);
     }
     __syncwarp();
     if ((tid & 31) == 0) mbar_arrive(empty);  // this warp is done with the stage
 
-    A drho[SPT], ux[SPT], uy[SPT], uz[SPT];
-    bool nonfinite = false;  // a density that is not finite or not positive
+    A r = f[0], j[3];
 #pragma unroll
-    for (int k = 0; k < SPT; k++) {
-        A r = A(0), jx = A(0), jy = A(0), jz = A(0);
+    for (int i = 1; i < kQ; i += 2) {
+        const A d = f[i] - f[i + 1];
+        r += f[i] + f[i + 1];
 #pragma unroll
-        for (int i = 0; i < kQ; i++) {
-            r += f[i][k];
-            if (cvec(i, 0)) jx += cvec(i, 0) * f[i][k];
-            if (cvec(i, 1)) jy += cvec(i, 1) * f[i][k];
-            if (cvec(i, 2)) jz += cvec(i, 2) * f[i][k];
+        for (int c = 0; c < 3; c++) {
+            if (i == 1 + 2 * c) j[c] = d;  // the axis pairs come first
+            else if (cvec(i, c) > 0) j[c] += d;
+            else if (cvec(i, c) < 0) j[c] -= d;
         }
-        const A rho = A(1) + r;
-        nonfinite |= !(rho > A(0) && rho < A(1e30));  // NaN fails both comparisons
-        const A inv = A(1) / rho;
-        if (ACCEL) {
-            jx += A(0.5) * rho * acA[0];
-            jy += A(0.5) * rho * acA[1];
-            jz += A(0.5) * rho * acA[2];
-        }
-        drho[k] = r;
-        ux[k] = jx * inv;
-        uy[k] = jy * inv;
-        uz[k] = jz * inv;
     }
-    // flag the box (it freezes from the next step on); boundary and inactive
-    // sites pulled zeros, so only collided sites can raise the flag
+    A rho = A(1) + r;
+    // flag the box (it freezes from the next step on) where a collided site's
+    // density is not finite or not positive; NaN fails both comparisons
+    const bool nonfinite = !(rho > A(0) && rho < A(1e30));
     if (__any_sync(0xffffffffu, nonfinite) && (tid & 31) == 0) atomicCAS(&p.status[th.box], 0, LB_ERR_NONFINITE);
+    A ac[3] = {A(0), A(0), A(0)};
+    if (ACCEL)
+        for (int c = 0; c < 3; c++) {
+            ac[c] = th.acc[c];
+            j[c] += A(0.5) * rho * ac[c];
+        }
+    const A inv = site_inverse(rho);
+    A ux = j[0] * inv, uy = j[1] * inv, uz = j[2] * inv;
+    A om = th.om, om1 = th.om1, sf = th.srcfac;
     // boundary sites: equilibrium of the boundary velocity from the ring
-    if (any_bnd) {
+    if (bnd) {
         TimeWeights<R> tw;
 #pragma unroll
         for (int a = 0; a < 4; a++) {
             tw.slot[a] = th.slot[a];
             tw.c[a] = th.c[a];
         }
-        const R* ring = reinterpret_cast<const R*>(p.ring);
-#pragma unroll
-        for (int k = 0; k < SPT; k++) {
-            if (bnd[k]) {
-                int pp, qq, x, y, z;
-                if (PER) {
-                    x = xs_[k];
-                    y = ys_[k];
-                    z = zs_[k];
-                } else {
-                    coords(k, x, y, z);
-                }
-                const int fc = owning_face(x, y, z, Ei, per, pp, qq);
-                float res[3];
-                load_mlp_residual(p, bd, th.mlp_s, fc, pp, qq, res);
-                R ub[3];
-                boundary_velocity<R>(ring, p.ring_slot_elems, bd, fc, pp, qq, tw, ub);
-                add_mlp_residual<R>(p, bd, res, ub);
-                drho[k] = th.drho_b;
-                ux[k] = (A)ub[0];
-                uy[k] = (A)ub[1];
-                uz[k] = (A)ub[2];
-            }
-        }
+        int pp, qq;
+        const int fc = owning_face(x, y, z, Ei, per, pp, qq);
+        float res[3];
+        load_mlp_residual(p, bd, th.mlp_s, fc, pp, qq, res);
+        R ub[3];
+        boundary_velocity<R>(reinterpret_cast<const R*>(p.ring), p.ring_slot_elems, bd, fc, pp, qq, tw, ub);
+        add_mlp_residual<R>(p, bd, res, ub);
+        r = th.drho_b;
+        rho = A(1) + r;
+        ux = (A)ub[0];
+        uy = (A)ub[1];
+        uz = (A)ub[2];
+        om = A(1);
+        om1 = sf = A(0);
     }
-    const A om = th.om, om1 = th.om1, srcfac = th.srcfac;
-    A usq[SPT], rho_[SPT], ua[SPT];
-#pragma unroll
-    for (int k = 0; k < SPT; k++) {
-        usq[k] = A(1.5) * (ux[k] * ux[k] + uy[k] * uy[k] + uz[k] * uz[k]);
-        rho_[k] = A(1) + drho[k];
-        if (ACCEL) ua[k] = ux[k] * acA[0] + uy[k] * acA[1] + uz[k] * acA[2];
+    const A xx = ux * ux, yy = uy * uy, zz = uz * uz;
+    // with k = om w rho, w = 1/18: om times the equilibrium of a pair is
+    // (w om drho - k 1.5 u^2) + k 4.5 cu^2 +- k 3 cu on an axis, half that on an edge
+    const A om18 = A(1) / A(18) * om, k18 = om18 * rho;
+    const A b18 = om18 * r - k18 * (A(1.5) * (xx + yy + zz)), b36 = A(0.5) * b18;
+    const A q18 = A(4.5) * k18, q36 = A(2.25) * k18, t18 = A(3) * k18, t36 = A(1.5) * k18;
+    A s18 = A(0), s36 = A(0), ua3 = A(0);
+    if (ACCEL) {
+        s18 = A(1) / A(18) * sf * rho;
+        s36 = A(0.5) * s18;
+        ua3 = A(-3) * (ux * ac[0] + uy * ac[1] + uz * ac[2]);
     }
-    // post-collision value of population i at site k from its equilibrium deviation
-    // populations are written in order 0, 1, ..., 18 through one running
-    // pointer (row of population i at this thread's first site)
-    E* out = Bb + s0 + tid;
-    auto emit = [&](int i, int k, A deq, A cu) {
-        A val = deq;
-        if (!bnd[k]) {
-            val = om1 * f[i][k] + om * deq;
-            if (ACCEL) {
-                const A w = wgt<A>(i);
-                A ca = A(0);  // c_i . a in the arithmetic type (FP64 is slow on this part)
-                if (cvec(i, 0)) ca += cvec(i, 0) * acA[0];
-                if (cvec(i, 1)) ca += cvec(i, 1) * acA[1];
-                if (cvec(i, 2)) ca += cvec(i, 2) * acA[2];
-                val += srcfac * w * rho_[k] * (A(3) * (ca - ua[k]) + A(9) * cu * ca);
-            }
-        }
-        // population 0 and odd i at `out`, the even partner of a pair one row further
-        const int row = (i > 0 && (i & 1) == 0) ? n3 : 0;
-        if (act[k]) st_stream(out + row + k * C, S::out(val));
-    };
-#pragma unroll
-    for (int k = 0; k < SPT; k++) emit(0, k, wgt<A>(0) * (drho[k] - rho_[k] * usq[k]), A(0));
-    // opposite pairs (1,2), (3,4), ..., (17,18)
+    // populations are written in order 0, 1, ..., 18 through one running pointer
+    E* out = Bb + s;
+    {
+        A val = om1 * f[0] + A(6) * b18;
+        if (ACCEL) val += A(6) * s18 * ua3;
+        if (act) st_stream(out, S::out(val));
+    }
 #pragma unroll
     for (int i = 1; i < kQ; i += 2) {
         out += i == 1 ? n3 : 2 * n3;  // row of population i; population i + 1 is one row further
-        const A w = wgt<A>(i);
         const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
-#pragma unroll
-        for (int k = 0; k < SPT; k++) {
-            A cu = A(0);
-            if (cx) cu += cx * ux[k];
-            if (cy) cu += cy * uy[k];
-            if (cz) cu += cz * uz[k];
-            const A even = w * (drho[k] + rho_[k] * (A(4.5) * cu * cu - usq[k]));
-            const A odd = (A(3) * w) * rho_[k] * cu;
-            emit(i, k, even + odd, cu);
-            emit(i + 1, k, even - odd, -cu);
+        const bool axis = i < 7;
+        // c_i . u of the first of the pair (an axis pair starts with the positive
+        // direction, an edge pair with its first component positive)
+        const A first = cx ? ux : (cy ? uy : uz), second = cz ? uz : uy;
+        const A cu = axis ? first : ((cx ? (cy ? cy : cz) : cz) > 0 ? first + second : first - second);
+        const A cu2 = axis ? (cx ? xx : (cy ? yy : zz)) : cu * cu;
+        A even = (axis ? q18 : q36) * cu2 + (axis ? b18 : b36);
+        A plus = even + (axis ? t18 : t36) * cu, minus = even - (axis ? t18 : t36) * cu;
+        if (ACCEL) {
+            A ca = A(0);  // c_i . a; c -> -c flips c.a and c.u
+            if (cx) ca += cx * ac[0];
+            if (cy) ca += cy * ac[1];
+            if (cz) ca += cz * ac[2];
+            const A sw = axis ? s18 : s36, e = A(9) * ca * cu + ua3;
+            plus += sw * (e + A(3) * ca);
+            minus += sw * (e - A(3) * ca);
+        }
+        if (act) {
+            st_stream(out, S::out(om1 * f[i] + plus));
+            st_stream(out + n3, S::out(om1 * f[i + 1] + minus));
         }
     }
 }
@@ -604,7 +564,7 @@ __device__ __forceinline__ void staged_tile_pair(const SCParams& p, const Staged
     if (__any_sync(0xffffffffu, nonfinite) && (tid & 31) == 0) atomicCAS(&p.status[th.box], 0, LB_ERR_NONFINITE);
     float2 ac[3] = {f2(0.f), f2(0.f), f2(0.f)};
     if (ACCEL) {
-        for (int c = 0; c < 3; c++) ac[c] = f2((float)bd.accel[c]);
+        for (int c = 0; c < 3; c++) ac[c] = f2(th.acc[c]);
         const float2 hr = mul2(f2(0.5f), rho);
         jx = fma2(hr, ac[0], jx);
         jy = fma2(hr, ac[1], jy);
@@ -700,9 +660,9 @@ __device__ __forceinline__ void staged_tile_pair(const SCParams& p, const Staged
         float2 vm = fma2(om1, f[i + 1], sub2(oeven, oodd));
         if (ACCEL) {
             float ca = 0.f;  // c_i . a (uniform per box)
-            if (cx) ca += cx * (float)bd.accel[0];
-            if (cy) ca += cy * (float)bd.accel[1];
-            if (cz) ca += cz * (float)bd.accel[2];
+            if (cx) ca += cx * ac[0].x;
+            if (cy) ca += cy * ac[1].x;
+            if (cz) ca += cz * ac[2].x;
             const float2 sw = w18 ? srcw[0] : srcw[1];
             // + : 3 (ca - ua) + 9 cu ca ;  - : 3 (-ca - ua) + 9 cu ca  (c -> -c flips ca and cu)
             const float2 nine_cu_ca = mul2(f2(9.f * ca), cu);
@@ -886,13 +846,13 @@ __device__ __forceinline__ void staged_consume(const SCParams& p, unsigned char*
                 else staged_tile_pair<ST, true, false>(p, th, stage, &hd->empty[st]);
             }
         } else if (!GENERAL) {
-            staged_tile<ST, SPT, false, false>(p, th, stage, &hd->empty[st]);
+            staged_tile<ST, false, false>(p, th, stage, &hd->empty[st]);
         } else if (bd.per_mask == 0) {
-            if (bd.has_accel) staged_tile<ST, SPT, false, true>(p, th, stage, &hd->empty[st]);
-            else staged_tile<ST, SPT, false, false>(p, th, stage, &hd->empty[st]);
+            if (bd.has_accel) staged_tile<ST, false, true>(p, th, stage, &hd->empty[st]);
+            else staged_tile<ST, false, false>(p, th, stage, &hd->empty[st]);
         } else {
-            if (bd.has_accel) staged_tile<ST, SPT, true, true>(p, th, stage, &hd->empty[st]);
-            else staged_tile<ST, SPT, true, false>(p, th, stage, &hd->empty[st]);
+            if (bd.has_accel) staged_tile<ST, true, true>(p, th, stage, &hd->empty[st]);
+            else staged_tile<ST, true, false>(p, th, stage, &hd->empty[st]);
         }
     }
 }
@@ -1089,6 +1049,7 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
                 th.om1 = A(1) - th.om;
                 th.srcfac = A(1) - A(0.5) * th.om;
                 th.drho_b = (A)th.bd.rho_b - A(1);
+                for (int c = 0; c < 3; c++) th.acc[c] = (A)th.bd.accel[c];
             }
             __syncwarp();
             Ei = th.bd.E;
