@@ -432,7 +432,7 @@ int enqueue_step(lb_ctx* ctx, int64_t n)
     fp.step = ctx->at<int64_t>(ctx->L.step);
     fp.tile_counter = ctx->at<int64_t>(ctx->L.tile_counter);
     fp.nchains = nch;
-    fp.splits = (8 * ctx->max_beads + kForcedThreads - 1) / kForcedThreads;
+    fp.splits = (8 * ctx->max_beads + forced_threads(ctx->storage) - 1) / forced_threads(ctx->storage);
     if (fp.splits < 1) fp.splits = 1;
     CK(DISPATCH(ctx->storage, forced(fp, ctx->stream)));
     ctx->a_is_pop_a = !ctx->a_is_pop_a;
@@ -685,6 +685,8 @@ int32_t lb_init(lb_ctx* ctx, int32_t box, const void* u0)
     }
     CK(DISPATCH(ctx->storage, init(A, ctx->boxes.data(), box, bd.n3, src, ctx->stream)));
     CK(cudaMemsetAsync(ctx->at<int32_t>(ctx->L.status) + box, 0, sizeof(int32_t), ctx->stream));
+    // no force list of an earlier run passes for one of the steps to come (k_forced)
+    CK(cudaMemsetAsync(ctx->at<double>(ctx->L.chain_accel), 0, sizeof(double) * 4 * (size_t)ctx->nboxes, ctx->stream));
     if (ctx->nboxes == 1) {
         ctx->step = 0;
         CK(cudaMemsetAsync(ctx->at<int64_t>(ctx->L.step), 0, sizeof(int64_t), ctx->stream));
@@ -1266,6 +1268,7 @@ int32_t lb_load(lb_ctx* ctx, const void* src)
     const int64_t step = h.step, zero = 0;
     CK(cudaMemcpyAsync(ctx->at<int64_t>(ctx->L.step), &step, sizeof step, cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->at<int64_t>(ctx->L.tile_counter), &zero, sizeof zero, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemsetAsync(ctx->at<double>(ctx->L.chain_accel), 0, sizeof(double) * 4 * (size_t)ctx->nboxes, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));  // host buffers above must outlive the copies
     ctx->step = step;
     ctx->pushed = pushed;

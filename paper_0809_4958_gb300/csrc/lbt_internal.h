@@ -17,7 +17,9 @@ constexpr int kMaxRingSlots = 4096;
 // points to cover site E - 1 (every site when z = 1).
 __host__ __device__ inline int coarse_points(int E, int z) { return z > 1 ? (E - 1 + z - 1) / z + 1 : E; }
 
-constexpr int kForcedThreads = 128;  // block of the forced re-collision (one force entry per thread)
+constexpr int kForcedThreads = 128;  // largest block of the forced re-collision (one force entry per thread)
+// its block for a storage format (0: FP64): single warps there, so that a chain's warps spread over SMs and their FP64 pipes
+__host__ __device__ constexpr int forced_threads(int storage) { return storage == 0 ? 32 : kForcedThreads; }
 constexpr int kMaxBeads = 256;      // beads per chain (one CTA per chain, one thread per bead)
 
 // One box as the kernels see it.
@@ -192,7 +194,7 @@ struct BeadParams {
     double* vel;
     ForceEntry* forces;
     const double* faccel;  // frame-acceleration samples [box][ring slot][4]
-    double* chain_accel;   // [chain][4]: the body acceleration of the step, for the forced sites
+    double* chain_accel;   // [chain][4]: the body acceleration of the step, for the forced sites; n + 1 (int64) behind it
     int32_t ring_slots;
     const int64_t* step;
     int32_t* status;
@@ -212,7 +214,7 @@ struct ForcedParams {
     const BoxDev* boxes;
     const ChainDev* chains;
     const ForceEntry* forces;
-    const double* chain_accel;    // [chain][4], written by the bead kernel of the step
+    const double* chain_accel;    // [chain][4], written by the bead kernel of the step (as in BeadParams)
     const int32_t* status;
     int64_t* step;                // incremented once per step by block 0
     int64_t* tile_counter;        // reset to zero once per step by block 0

@@ -242,7 +242,42 @@ __global__ void __launch_bounds__(256) k_stream_collide(SCParams p)
 // Per-site helpers for the scalar kernels (bead gather, forced re-collision,
 // fields).
 // ---------------------------------------------------------------------------
-template <int ST>
+// j / rho from r = 1 / rho, the product corrected by its own residual (within
+// one ulp), so that the three components share one reciprocal; the division
+// itself where the result is not finite.
+static __device__ __noinline__ double slow_ratio(double j, double rho) { return j / rho; }
+static __device__ __noinline__ float slow_ratio(float j, float rho) { return j / rho; }
+template <class A>
+__device__ __forceinline__ A ratio(A j, A rho, A r)
+{
+    const A q = j * r, t = fma(fma(-q, rho, j), r, q);
+    return isfinite(t) ? t : slow_ratio(j, rho);
+}
+// Density deviation and (WHAT = 1) momentum of one site from its populations,
+// by opposite pairs: their sums make the density, their differences the
+// momentum (39 additions in place of 48).
+template <class A, int WHAT, class F>
+__device__ __forceinline__ void site_moments(const F& f, A& r, A j[3])
+{
+    r = f(0);
+#pragma unroll
+    for (int i = 1; i < kQ; i += 2) {
+        const A a = f(i), b = f(i + 1);
+        r += a + b;
+        if (WHAT == 1) {
+            const A d = a - b;
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                if (i == 1 + 2 * c) j[c] = d;  // the axis pairs come first
+                else if (cvec(i, c) > 0) j[c] += d;
+                else if (cvec(i, c) < 0) j[c] -= d;
+            }
+        }
+    }
+}
+
+// (L2: read past L1)
+template <int ST, bool L2 = false>
 __device__ __forceinline__ void pull_site(const typename Stor<ST>::E* Ab, int64_t n3, int E, int per, int x, int y,
                                           int z, typename Stor<ST>::A f[kQ])
 {
@@ -252,7 +287,8 @@ __device__ __forceinline__ void pull_site(const typename Stor<ST>::E* Ab, int64_
         if (per & 1) xs = wrapi(xs, E);
         if (per & 2) ys = wrapi(ys, E);
         if (per & 4) zs = wrapi(zs, E);
-        f[i] = Stor<ST>::in(Ab[(int64_t)i * n3 + ((int64_t)zs * E + ys) * E + xs]);
+        const typename Stor<ST>::E* src = Ab + (int64_t)i * n3 + ((int64_t)zs * E + ys) * E + xs;
+        f[i] = Stor<ST>::in(L2 ? __ldcg(src) : *src);
     }
 }
 
@@ -288,6 +324,7 @@ constexpr int kMaxStencilNb = 24;       // listed beads with a nearby stencil (m
 constexpr int kNoiseChunk = 64;         // substeps whose noise is drawn at once (at most)
 constexpr int kBeadThreadsMax = 2 * kMaxBeads;  // 512: two MD lanes per bead at the largest chain
 constexpr size_t kBeadDynMax = 160 * 1024;      // dynamic shared memory budget of the bead kernel
+constexpr size_t kBeadDynShared = 64 * 1024;    // ... where two blocks share an SM (with 43 KB static each)
 
 template <class MT>
 struct Vec4;
@@ -306,19 +343,19 @@ struct Vec4<double> {
 // substeps (at most kNoiseChunk) as fit the dynamic shared-memory budget next
 // to the two position buffers, all 4-vectors.
 template <class MT>
-inline int bead_noise_chunk(int maxb)
+inline int bead_noise_chunk(int maxb, size_t budget)
 {
     const size_t per = 4 * sizeof(MT) * (size_t)(maxb > 0 ? maxb : 1);
-    const int c = (int)(kBeadDynMax / per) - 2;
+    const int c = (int)(budget / per) - 2;
     return c < kNoiseChunk ? (c < 1 ? 1 : c) : kNoiseChunk;
 }
 
 // Dynamic shared memory: positions relative to bead 0's start-of-step
 // position, double-buffered over substeps, and the noise of one chunk.
 template <class MT>
-inline size_t bead_dyn_bytes(int maxb)
+inline size_t bead_dyn_bytes(int maxb, size_t budget)
 {
-    return 4 * sizeof(MT) * (size_t)maxb * (2 + bead_noise_chunk<MT>(maxb));
+    return 4 * sizeof(MT) * (size_t)maxb * (2 + bead_noise_chunk<MT>(maxb, budget));
 }
 
 // Pair-force constants of a chain in the MD precision.
@@ -1130,10 +1167,10 @@ __global__ void __launch_bounds__(kBeadThreadsMax) k_bead_couple(BeadParams p)
     // 3. MD substeps (md_substeps below)
     {
         __shared__ int sErrP[2];
-        int err;
-        if (p.beads_per_thread == 0)
+        int err = 0;
+        if (p.beads_per_thread == 0) {
             err = md_chain_pairs<MT>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
-        else if (p.beads_per_thread == 1 && p.lanes == 8)
+        } else if (p.beads_per_thread == 1 && p.lanes == 8)
             err = md_substeps_split<MT, 8>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
         else if (p.beads_per_thread == 1 && p.lanes == 4)
             err = md_substeps_split<MT, 4>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
@@ -1273,6 +1310,14 @@ __global__ void __launch_bounds__(kBeadThreadsMax) k_bead_couple(BeadParams p)
         for (int a = 0; a < 3; a++) fe.g[a] = (double)g[a];
         fl[e] = fe;
     }
+    // the list of step n is complete (k_forced may read it now)
+    __syncthreads();
+    if (tid == 0) {
+        const int64_t mark = n + 1;
+        asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(reinterpret_cast<int64_t*>(p.chain_accel + 4 * blockIdx.x + 3)),
+                     "l"(mark)
+                     : "memory");
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1286,52 +1331,90 @@ __global__ void __launch_bounds__(kForcedThreads) k_forced(ForcedParams p)
     // the next step's stream-collide (a programmatic dependent) may be
     // scheduled now; it waits on the device for this kernel to complete
     asm volatile("griddepcontrol.launch_dependents;");
-    // this kernel is itself a programmatic dependent of the stream-collide
-    // before it: wait for that grid to complete and its stores to be visible
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // This kernel is itself a programmatic dependent of the stream-collide
+    // before it and may run while that one finishes its last tiles.  Its input
+    // is the state A both read and the bead kernel's force list; the bead block
+    // of a chain, which itself ran behind everything that wrote A, marks the
+    // list of step n with n + 1 (released, acquired here).  Where the mark is
+    // there, the new populations are worked out at once and only the stores wait
+    // for the stream-collide, which writes the same sites; otherwise everything
+    // waits (128^3 FP32 with a 64-bead chain: 59.8 -> 58.6 us a step).
     using S = Stor<ST>;
     using A = typename S::A;
-    const int chain = (int)blockIdx.x / p.splits, part = (int)blockIdx.x - chain * p.splits;
-    if (chain < p.nchains) {
-        const ChainDev& ch = p.chains[chain];
-        const int b = ch.box, nb = ch.nbeads;
-        const ForceEntry* fl = p.forces + ch.force_off;
-        // the entry, the status and the box record are independent loads:
-        // issue them together (e stays inside the chain's entries)
-        for (int e = part * blockDim.x + threadIdx.x; e < 8 * nb; e += p.splits * blockDim.x) {
-            const ForceEntry fe = fl[e];
-            const int st = p.status[b];
-            const BoxDev& bd = p.boxes[b];
+    const int chain = (int)blockIdx.x / p.splits;
+    const int e = ((int)blockIdx.x - chain * p.splits) * (int)blockDim.x + (int)threadIdx.x;  // one entry a thread
+    const bool mine = chain < p.nchains && e < 8 * p.chains[chain].nbeads;
+    bool ready = false;
+    if (mine) {
+        const int64_t n = *reinterpret_cast<const volatile int64_t*>(p.step);
+        int64_t mark;
+        asm volatile("ld.acquire.gpu.global.b64 %0, [%1];"
+                     : "=l"(mark)
+                     : "l"(reinterpret_cast<const int64_t*>(p.chain_accel + 4 * chain + 3))
+                     : "memory");
+        ready = mark == n + 1;
+    }
+    A val[kQ];
+    int site = -1;
+    typename S::E* Bb = nullptr;
+    int64_t n3 = 0;
+    bool clean = true;  // the box carries no error status
+#pragma unroll 1
+    for (int pass = 0; pass < 2; pass++) {
+        if (pass == 1) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");  // that grid complete and its stores visible
+            clean = mine && *reinterpret_cast<const volatile int32_t*>(p.status + p.chains[chain].box) == 0;
+        }
+        if (mine && (pass == 0 ? ready : clean && !ready)) {
+            const ChainDev& ch = p.chains[chain];
+            const BoxDev& bd = p.boxes[ch.box];
+            const ForceEntry fe = p.forces[ch.force_off + e];
             const int Ei = bd.E, per = bd.per_mask;
-            const int64_t n3 = bd.n3;
+            n3 = bd.n3;
             const typename S::E* Ab = reinterpret_cast<const typename S::E*>(p.A) + bd.f_off;
-            typename S::E* Bb = reinterpret_cast<typename S::E*>(p.B) + bd.f_off;
-            if (fe.site < 0 || st != 0) continue;
-            const int x = fe.site % Ei, y = (fe.site / Ei) % Ei, z = fe.site / (Ei * Ei);
-            A f[kQ], dr, j[3];
-            pull_site<ST>(Ab, n3, Ei, per, x, y, z, f);
-            moments<A>(f, dr, j);
-            const A rho = A(1) + dr;
-            A F[3], u[3];
-            for (int a = 0; a < 3; a++) {
-                F[a] = rho * (A)p.chain_accel[4 * chain + a] + (A)fe.g[a];
-                u[a] = (j[a] + A(0.5) * F[a]) / rho;
-            }
-            const A om = A(1) / (A)bd.tau;
-            const A usq = A(1.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-            const A uF = u[0] * F[0] + u[1] * F[1] + u[2] * F[2];
+            Bb = reinterpret_cast<typename S::E*>(p.B) + bd.f_off;
+            if (fe.site >= 0) {
+                site = fe.site;
+                const int x = site % Ei, y = (site / Ei) % Ei, z = site / (Ei * Ei);
+                A dr, j[3];
+                pull_site<ST, true>(Ab, n3, Ei, per, x, y, z, val);
+                site_moments<A, 1>([&](int i) { return val[i]; }, dr, j);
+                const A rho = A(1) + dr, inv = fast_inverse(rho);
+                A F[3], u[3];
+                for (int a = 0; a < 3; a++) {
+                    F[a] = rho * (A)p.chain_accel[4 * chain + a] + (A)fe.g[a];
+                    u[a] = ratio(j[a] + A(0.5) * F[a], rho, inv);
+                }
+                const A om = A(1) / (A)bd.tau, om1 = A(1) - om, sf = A(1) - A(0.5) * om;
+                const A usq = A(1.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+                const A uF3 = A(3) * (u[0] * F[0] + u[1] * F[1] + u[2] * F[2]);
+                // by opposite pairs: om (drho + rho (4.5 cu^2 - 1.5 u^2)) + sf (9 cu cF - 3 u.F) in common,
+                // om rho 3 cu + sf 3 cF changing sign
+                const A even0 = om * (dr - rho * usq) - sf * uF3, omr = om * rho;
+                val[0] = om1 * val[0] + wgt<A>(0) * even0;
 #pragma unroll
-            for (int i = 0; i < kQ; i++) {
-                const A w = wgt<A>(i);
-                const A cu = cvec(i, 0) * u[0] + cvec(i, 1) * u[1] + cvec(i, 2) * u[2];
-                const A cF = cvec(i, 0) * F[0] + cvec(i, 1) * F[1] + cvec(i, 2) * F[2];
-                const A deq = w * (dr + rho * (A(3) * cu + A(4.5) * cu * cu - usq));
-                A val = f[i] + om * (deq - f[i]);
-                val += (A(1) - A(0.5) * om) * w * (A(3) * (cF - uF) + A(9) * cu * cF);
-                Bb[(int64_t)i * n3 + fe.site] = S::out(val);
+                for (int i = 1; i < kQ; i += 2) {
+                    A cu = A(0), cF = A(0);
+                    bool some = false;
+#pragma unroll
+                    for (int a = 0; a < 3; a++)
+                        if (cvec(i, a)) {
+                            const A su = cvec(i, a) > 0 ? u[a] : -u[a], sF = cvec(i, a) > 0 ? F[a] : -F[a];
+                            cu = some ? cu + su : su;
+                            cF = some ? cF + sF : sF;
+                            some = true;
+                        }
+                    const A w = wgt<A>(i);
+                    const A even = even0 + cu * (A(4.5) * omr * cu + A(9) * sf * cF), odd = A(3) * (omr * cu + sf * cF);
+                    val[i] = om1 * val[i] + w * (even + odd);
+                    val[i + 1] = om1 * val[i + 1] + w * (even - odd);
+                }
             }
         }
     }
+    if (clean && site >= 0)
+#pragma unroll
+        for (int i = 0; i < kQ; i++) Bb[(int64_t)i * n3 + site] = S::out(val[i]);
     if (blockIdx.x == 0) {
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -1408,40 +1491,6 @@ __global__ void k_init(typename Stor<ST>::E* Ab, BoxDev bd, const typename Stor<
 // shuffles in FP64 140 / 302.
 // ---------------------------------------------------------------------------
 constexpr int kFieldsThreads = 256;
-
-// j / rho from r = 1 / rho, the product corrected by its own residual (within
-// one ulp), so that the three components share one reciprocal; the division
-// itself where the result is not finite.
-static __device__ __noinline__ double slow_ratio(double j, double rho) { return j / rho; }
-static __device__ __noinline__ float slow_ratio(float j, float rho) { return j / rho; }
-template <class A>
-__device__ __forceinline__ A ratio(A j, A rho, A r)
-{
-    const A q = j * r, t = fma(fma(-q, rho, j), r, q);
-    return isfinite(t) ? t : slow_ratio(j, rho);
-}
-// Density deviation and (WHAT = 1) momentum of one site from its populations,
-// by opposite pairs: their sums make the density, their differences the
-// momentum (39 additions in place of 48).
-template <class A, int WHAT, class F>
-__device__ __forceinline__ void site_moments(const F& f, A& r, A j[3])
-{
-    r = f(0);
-#pragma unroll
-    for (int i = 1; i < kQ; i += 2) {
-        const A a = f(i), b = f(i + 1);
-        r += a + b;
-        if (WHAT == 1) {
-            const A d = a - b;
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                if (i == 1 + 2 * c) j[c] = d;  // the axis pairs come first
-                else if (cvec(i, c) > 0) j[c] += d;
-                else if (cvec(i, c) < 0) j[c] -= d;
-            }
-        }
-    }
-}
 
 // The value of lane - 1 (up) or lane + 1.
 template <class E>
@@ -1746,13 +1795,23 @@ cudaError_t Launch<ST>::bead_couple(const BeadParams& p, int nchains, int max_be
 {
     if (nchains <= 0) return cudaSuccess;
     using MT = typename std::conditional<ST == kF64, double, float>::type;
-    const size_t dyn = bead_dyn_bytes<MT>(max_beads);
+    // More chains than SMs: a block is latency bound and its SM is closed to
+    // the stream-collide meanwhile, so two share an SM -- blocks of 256 threads
+    // (128 registers each) and at most kBeadDynShared bytes of noise and
+    // positions.  512 chains of up to 96 beads next to their boxes:
+    // 1497 -> 1464 us a step.
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const bool share = sizeof(MT) == 4 && nchains > sms && lanes <= 0;
+    const size_t budget = share ? kBeadDynShared : kBeadDynMax;
+    const size_t dyn = bead_dyn_bytes<MT>(max_beads, budget);
     static int attr_done[kMaxDevices] = {};  // largest dynamic size enabled so far, per device
     cudaError_t e = smem_attr_per_device(k_bead_couple<ST>, (int)dyn, attr_done);
     if (e != cudaSuccess) return e;
     BeadParams q = p;
     q.max_beads = max_beads;
-    q.noise_chunk = bead_noise_chunk<MT>(max_beads);
+    q.noise_chunk = bead_noise_chunk<MT>(max_beads, budget);
     // MD layout (validated by the caller): lanes per bead and beads per
     // thread; 0 = default, the chain-order layout (two lanes per bead; the
     // autotuner's choice for the 64-bead chain of the 128^3 box: 0.0655 ms per
@@ -1769,7 +1828,7 @@ cudaError_t Launch<ST>::bead_couple(const BeadParams& p, int nchains, int max_be
     int threads = bpt == 0 ? 8 * max_beads : lanes * ((max_beads + bpt - 1) / bpt);
     threads = (threads + 31) / 32 * 32;
     if (threads > kBeadThreadsMax) threads = kBeadThreadsMax;
-    if (threads < 256) threads = 256;
+    if (threads < 256 || (share && 2 * max_beads <= 256)) threads = 256;
     k_bead_couple<ST><<<nchains, threads, dyn, s>>>(q);
     return cudaGetLastError();
 }
@@ -1806,7 +1865,7 @@ cudaError_t Launch<ST>::forced(const ForcedParams& p, cudaStream_t s)
     // device for it to complete)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.nchains > 0 ? p.nchains * p.splits : 1));
-    cfg.blockDim = dim3(kForcedThreads);
+    cfg.blockDim = dim3(forced_threads(ST));
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
