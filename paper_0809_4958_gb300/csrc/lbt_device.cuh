@@ -148,8 +148,10 @@ __device__ __forceinline__ T unit_uniform_t(uint32_t v);
 template <>
 __device__ __forceinline__ double unit_uniform_t<double>(uint32_t v)
 {
-    const double u01 = (double)v * (1.0 / 4294967296.0);  // 2^-32
-    return sqrt(3.0) * (2.0 * u01 - 1.0);
+    // 1 + v 2^-32 by placing the bits (a conversion runs on the FP64 pipe, two
+    // lanes a clock); 2 (1 + v 2^-32) - 3 = 2 v 2^-32 - 1 is exact
+    const double x = __hiloint2double((int)(0x3ff00000u | (v >> 12)), (int)(v << 20));
+    return sqrt(3.0) * fma(2.0, x, -3.0);
 }
 template <>
 __device__ __forceinline__ float unit_uniform_t<float>(uint32_t v)
@@ -176,20 +178,10 @@ __device__ __forceinline__ float fast_inverse(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// Reciprocal of the bead pair forces: correctly rounded division in FP64,
-// the hardware's approximate reciprocal in FP32 (PTX rcp.approx.ftz.f32, at
-// most one ulp off, far below the FP32 dynamics' own rounding; the pair
-// arguments are never subnormal).  One instruction: the MD substeps are a
-// latency-bound chain, and the approximate division intrinsic it replaces
-// cost half of a substep's force phase.
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
-__device__ __forceinline__ float recip(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
+// Reciprocal of the bead pair forces, whose arguments are never subnormal: the
+// MD substeps are a latency-bound chain.
+__device__ __forceinline__ double recip(double x) { return fast_inverse(x); }
+__device__ __forceinline__ float recip(float x) { return fast_inverse(x); }
 // 1 / rho of a collided site: in FP64 by fast_inverse (the FP64 pipe bounds
 // that collision), the division in FP32.
 __device__ __forceinline__ double site_inverse(double rho) { return fast_inverse(rho); }

@@ -323,7 +323,7 @@ constexpr int kMaxTasks = 48;           // pair tasks (bonds + Verlet neighbours
 constexpr int kMaxStencilNb = 24;       // listed beads with a nearby stencil (more: scan all)
 constexpr int kNoiseChunk = 64;         // substeps whose noise is drawn at once (at most)
 constexpr int kBeadThreadsMax = 2 * kMaxBeads;  // 512: two MD lanes per bead at the largest chain
-constexpr size_t kBeadDynMax = 160 * 1024;      // dynamic shared memory budget of the bead kernel
+constexpr size_t kBeadDynMax = 144 * 1024;      // dynamic shared memory budget of the bead kernel
 constexpr size_t kBeadDynShared = 64 * 1024;    // ... where two blocks share an SM (with 43 KB static each)
 
 template <class MT>
@@ -1038,6 +1038,226 @@ __device__ __forceinline__ int md_chain_pairs(const BeadParams& p, const ChainDe
     return 0;
 }
 
+// The chain-order substeps in FP64, four warps to 32 beads.  An FP64
+// instruction of a warp holds its quarter of the SM for 64 cycles, however many
+// lanes work, so what counts is how many of them the busiest quarter runs.
+// Every pair near along the chain is evaluated once, a lane per bead g, and the
+// work is split by role: warp role 0 the bonds (g, g + 1) (FENE and WCA), role 1
+// the pairs (g, g + 2) (WCA), roles 2 and 3 the even and odd entries of the
+// Verlet lists of the pairs at least three apart (from both their beads, the law
+// skipped where no lane is within the cut-off).  The forces meet in shared
+// memory; then roles 0 - 2 advance component x, y and z of every bead.  Two
+// barriers a substep.  Groups of 32 beads rotate the roles over the quarters.
+// Lists come from FP32 copies of the positions with a radius larger by 1e-5,
+// more than their rounding: a superset, and a pair beyond the cut-off adds
+// exactly zero.  (All of a bead's work in one lane: 202 us a step of the 16-bead
+// chain in a 32^3 box and 247 of 64 beads; two lanes a bead with masked slots
+// and divisions: 298 and 371; ROLES_US.)  Flags and errors as in md_chain_pairs.
+constexpr int kRoleBeads = kBeadThreadsMax / 4;  // beads the four roles' warps cover
+
+__device__ __forceinline__ int md_chain_roles(const BeadParams& p, const ChainDev& ch, int N, int64_t n, int b,
+                                              double* sXbuf, double (*sU)[3], double (*sV)[3], double (*sR)[3],
+                                              double (*sP)[3], unsigned char (*sNb)[kMaxTasks], int* sErrP)
+{
+    using V4 = typename Vec4<double>::T;
+    __shared__ int sNbN[kRoleBeads];  // listed partners of each bead
+    __shared__ float4 sXf[kRoleBeads];
+    __shared__ double sF[4][3][kRoleBeads + 2];  // role, component, bead + 2 (two zeros in front)
+    __shared__ int sErrB;             // list overflow of the block's build
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int maxb = p.max_beads;
+    V4* sX4 = reinterpret_cast<V4*>(sXbuf);  // [2][maxb] positions, then [chunk][N] noise
+    const double* sXi = reinterpret_cast<const double*>(sX4 + 2 * maxb);
+    const double* mc = ch.md_d;
+    const double dt = mc[kMdDt], dtm = mc[kMdDtm], namp = mc[kMdNamp], zeta = mc[kMdZeta];
+    const double R02 = mc[kMdR02], invR02 = mc[kMdInvR02], kf = mc[kMdKf], sig2 = mc[kMdSig2], rc2 = mc[kMdRc2],
+                 e24 = mc[kMdE24];
+    const bool wca = ch.eps > 0.0;
+    const float rl2 = (float)mc[kMdRl2] * (1.0f + 2e-5f);
+    const double skin_c2 = mc[kMdSkinComp2];
+    if (tid < 2) sErrP[tid] = 0;
+    if (tid == 0) sErrB = 0;
+    for (int g = tid; g < N; g += nthr) sXf[g] = make_float4((float)sX4[g].x, (float)sX4[g].y, (float)sX4[g].z, 0.f);
+    for (int e = tid; e < 4 * 3 * (kRoleBeads + 2); e += nthr) (&sF[0][0][0])[e] = 0.0;
+    __syncthreads();
+    // lists from the start positions: eight threads per bead scan every eighth partner and merge
+    // their finds in order by a prefix sum over the eight
+    if (wca) {
+        for (int base = 0; base < 8 * N; base += nthr) {
+            const int e = base + tid;
+            const bool act = e < 8 * N;
+            const int bb = act ? e >> 3 : 0, r = e & 7;
+            uint32_t m = 0;  // bit k: partner r + 8 k (N <= 256)
+            if (act) {
+                const float4 xb = sXf[bb];
+                for (int k = 0, p2 = r; p2 < N; k++, p2 += 8) {
+                    const int dd = p2 - bb;
+                    if (dd >= -2 && dd <= 2) continue;
+                    const float4 q = sXf[p2];
+                    const float dx = xb.x - q.x, dy = xb.y - q.y, dz = xb.z - q.z;
+                    if (dx * dx + dy * dy + dz * dz < rl2) m |= 1u << k;
+                }
+            }
+            const int cnt = __popc(m);
+            int incl = cnt;
+            for (int o = 1; o < 8; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o, 8);
+                if (r >= o) incl += v;
+            }
+            const int total = __shfl_sync(0xffffffffu, incl, 7, 8);
+            if (act) {
+                int k = incl - cnt;
+                for (uint32_t mm = m; mm; mm &= mm - 1, k++)
+                    if (k < kMaxTasks) sNb[bb][k] = (unsigned char)(r + 8 * (__ffs(mm) - 1));
+                if (r == 7) {
+                    sNbN[bb] = total;
+                    if (total > kMaxTasks) sErrB = LB_ERR_CHAIN;  // more neighbours than the list holds
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (sErrB) return sErrB;
+
+    const int nmd = 128 * ((N + 31) / 32);  // MD threads
+    const bool md = tid < nmd;
+    const int group = tid >> 7, role = ((tid >> 5) + group) & 3;
+    const int g = 32 * group + (tid & 31);  // bead of this lane
+    const bool own = md && g < N;
+    const int i0 = own ? g : 0;
+    // force roles: the partner (roles 0, 1) or the list (2, 3)
+    const bool on = own && (role == 0 ? g + 1 < N : g + 2 < N && wca);
+    const int i1 = role < 2 && on ? g + 1 + role : i0;
+    int nl = 0, kmax = 0;  // entries of this role's half of the list, and the warp's largest
+    auto load_list = [&]() {
+        const int all = own && wca ? min(sNbN[i0], kMaxTasks) : 0;
+        nl = role == 2 ? (all + 1) >> 1 : (role == 3 ? all >> 1 : 0);
+        kmax = __reduce_max_sync(0xffffffffu, nl);
+    };
+    if (md) load_list();
+    // update roles: component c of the bead
+    const int c = role < 3 ? role : 0;
+    const bool upd = own && role < 3;
+    const double x0 = sXbuf[4 * i0 + c], zu = zeta * sU[i0][c], fx = ch.f_ext[c];
+    double v = sV[i0][c], d = 0.0, pm = 0.0, dref = 0.0;
+    // 24 eps (2 (s/r)^12 - (s/r)^6) / r^2
+    auto wca_fac = [&](double r2) {
+        const double inv = recip(r2), s2 = sig2 * inv, s6 = s2 * s2 * s2;
+        return fma(2.0, s6, -1.0) * s6 * (e24 * inv);
+    };
+    auto sync_md = [&](int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nmd) : "memory"); };
+    const int chunk = namp > 0.0 ? p.noise_chunk : ch.n_md;
+    for (int c0 = 0; c0 < ch.n_md; c0 += chunk) {
+        const int nc = min(chunk, ch.n_md - c0);
+        if (namp > 0.0) {
+            __syncthreads();  // the previous chunk's noise is consumed
+            md_noise<double>(sX4 + 2 * maxb, n, c0, nc, N, b, ch.seed);
+            __syncthreads();
+        }
+        if (md) {
+            for (int sb = 0; sb < nc; sb++) {
+                const int sub = c0 + sb;
+                const V4* Xc = sX4 + (sub & 1) * maxb;
+                double* Xn = sXbuf + 4 * ((sub + 1) & 1) * maxb;
+                bool stretched = false;
+                {
+                    const V4 x = Xc[i0];
+                    double f[3];
+                    if (role < 2) {
+                        const V4 q = Xc[i1];
+                        const double ax = x.x - q.x, ay = x.y - q.y, az = x.z - q.z;
+                        const double r2 = ax * ax + ay * ay + az * az;
+                        double h = 0.0;
+                        if (role == 0) {
+                            h = -kf * recip(1.0 - r2 * invR02);
+                            stretched = on && r2 >= R02;
+                        }
+                        const bool near = on && wca && r2 < rc2;
+                        if (__any_sync(0xffffffffu, near)) {
+                            const double w = wca_fac(r2);
+                            h += near ? w : 0.0;
+                        }
+                        h = on ? h : 0.0;
+                        f[0] = h * ax;
+                        f[1] = h * ay;
+                        f[2] = h * az;
+                    } else {
+                        f[0] = f[1] = f[2] = 0.0;
+                        for (int s = 0; s < kmax; s++) {
+                            const V4 q = Xc[s < nl ? sNb[i0][2 * s + role - 2] : i0];
+                            const double ax = x.x - q.x, ay = x.y - q.y, az = x.z - q.z;
+                            const double r2 = ax * ax + ay * ay + az * az;
+                            const bool near = s < nl && r2 < rc2;
+                            if (__any_sync(0xffffffffu, near)) {
+                                const double w = wca_fac(r2), h = near ? w : 0.0;
+                                f[0] += h * ax;
+                                f[1] += h * ay;
+                                f[2] += h * az;
+                            }
+                        }
+                    }
+                    if (own)
+#pragma unroll
+                        for (int a = 0; a < 3; a++) sF[role][a][g + 2] = f[a];
+                }
+                sync_md(2);
+                bool moved = false;
+                if (role < 3) {  // whole warps
+                    // the force of a pair on its second bead is the first one's, negated
+                    const double F = ((sF[0][c][i0 + 2] - sF[0][c][i0 + 1]) + (sF[1][c][i0 + 2] - sF[1][c][i0])) +
+                                     (sF[2][c][i0 + 2] + sF[3][c][i0 + 2]);
+                    const double ff = fma(-zeta, v, namp > 0.0 ? fma(namp, sXi[4 * (sb * N + i0) + c], zu) : zu);  // friction, noise
+                    v = fma(dtm, F + (ff + fx), v);
+                    d = fma(dt, v, d);
+                    if (upd) Xn[4 * g + c] = x0 + d;
+                    pm = fma(-dt, ff, pm);
+                    const double dm = d - dref;
+                    moved = upd && wca && dm * dm > skin_c2;
+                }
+                if (stretched) sErrP[sub & 1] = LB_ERR_FENE;
+                // publish Xn; any flag: stop on an error, or rebuild the lists
+                if (bar_or(1, nmd, stretched || moved)) {
+                    if (sErrP[sub & 1]) break;
+                    if (own && role == 3) sXf[g] = make_float4((float)Xn[4 * g], (float)Xn[4 * g + 1], (float)Xn[4 * g + 2], 0.f);
+                    sync_md(2);
+                    if (own && role == 2 && wca) {
+                        const float4 xb = sXf[g];
+                        int cnt = 0;
+                        for (int p2 = 0; p2 < N; p2++) {
+                            const int dd = p2 - g;
+                            if (dd >= -2 && dd <= 2) continue;
+                            const float4 q = sXf[p2];
+                            const float ex = xb.x - q.x, ey = xb.y - q.y, ez = xb.z - q.z;
+                            if (ex * ex + ey * ey + ez * ez < rl2) {
+                                if (cnt < kMaxTasks) sNb[g][cnt] = (unsigned char)p2;
+                                cnt++;
+                            }
+                        }
+                        sNbN[g] = cnt;
+                        // more neighbours than the list holds: the error stops
+                        // the next barrier (or the chunk's)
+                        if (cnt > kMaxTasks) sErrP[(sub + 1) & 1] = LB_ERR_CHAIN;
+                    }
+                    sync_md(2);
+                    load_list();
+                    dref = d;
+                }
+            }
+        }
+        __syncthreads();
+        if (sErrP[0] || sErrP[1]) break;
+    }
+    const int err = sErrP[0] ? sErrP[0] : sErrP[1];
+    if (err) return err;
+    if (upd) {
+        sR[g][c] += d;
+        sV[g][c] = v;
+        sP[g][c] = pm;
+    }
+    __syncthreads();
+    return 0;
+}
+
 template <int ST>
 __global__ void __launch_bounds__(kBeadThreadsMax) k_bead_couple(BeadParams p)
 {
@@ -1169,7 +1389,12 @@ __global__ void __launch_bounds__(kBeadThreadsMax) k_bead_couple(BeadParams p)
         __shared__ int sErrP[2];
         int err = 0;
         if (p.beads_per_thread == 0) {
-            err = md_chain_pairs<MT>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
+            bool roles = false;
+            if constexpr (sizeof(MT) == 8) {
+                roles = N <= kRoleBeads && nthr >= 128 * ((N + 31) / 32);
+                if (roles) err = md_chain_roles(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
+            }
+            if (!roles) err = md_chain_pairs<MT>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
         } else if (p.beads_per_thread == 1 && p.lanes == 8)
             err = md_substeps_split<MT, 8>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
         else if (p.beads_per_thread == 1 && p.lanes == 4)
