@@ -1299,6 +1299,8 @@ int32_t lb_set_fluctuation(lb_ctx* ctx, int32_t box, double kT, uint64_t seed, c
             const double b = bnorm36(k) / 36.0;
             fd.gamma[k - 4] = gamma[k];
             fd.amp[k - 4] = std::sqrt(3.0 * kT * b * (1.0 - gamma[k] * gamma[k]));
+            fd.gamma_f[k - 4] = (float)(fd.gamma[k - 4] / b);
+            fd.amp_f[k - 4] = (float)(fd.amp[k - 4] / b);
         }
     }
     bd.fluct = fd.on;

@@ -112,6 +112,9 @@ struct FluctDev {
     int32_t pad;
     double gamma[15];  // relaxation factor of modes 4 .. 18
     double amp[15];    // sqrt(3 kT b_k (1 - gamma_k^2)); times sqrt(rho) per site
+    // both over b_k, in FP32, for the packed FP32 collision (16th entry unused)
+    alignas(16) float gamma_f[16];
+    alignas(16) float amp_f[16];
 };
 
 // Force density at one lattice site, produced by the bead kernel, consumed by

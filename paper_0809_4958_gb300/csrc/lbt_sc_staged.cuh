@@ -472,6 +472,53 @@ __device__ __forceinline__ void edge_velocity(const SCParams& p, const StagedTil
         for (int c = 0; c < 3; c++) u[c] += p.mlp_yunit * e[c * st];
 }
 
+// Velocity and density deviation of the boundary sites among a thread's
+// adjacent pair (x, x + 1) of box row `row` = (y, z): ue is the x-face site's
+// velocity where the tile's samples were staged (staged), else it is loaded here.
+template <int ST>
+__device__ __forceinline__ void boundary_pair(const SCParams& p, const StagedTile<ST>& th, int row, int x, int y, int z,
+                                              bool brow, bool xface0, bool xface1, bool staged, float ue[3], float2& ux,
+                                              float2& uy, float2& uz, float2& drho)
+{
+    const BoxDev& bd = th.bd;
+    const int Ei = bd.E;
+    const bool py = bd.per_mask & 2;
+    if (brow) {  // a row on a y or z face (its x-face sites, which belong to the x faces, follow)
+        const int f = !py && y == 0 ? 2 : (!py && y == Ei - 1 ? 3 : (z == 0 ? 4 : 5));
+        float2 u[3];
+        boundary_velocity_pair(p, th, f, f < 4 ? z : y, x, u);
+        ux = u[0];
+        uy = u[1];
+        uz = u[2];
+        drho = f2(th.drho_b);
+    }
+    if (xface0 || xface1) {
+        if (!staged) {
+            TimeWeights<float> tw;
+#pragma unroll
+            for (int a = 0; a < 4; a++) {
+                tw.slot[a] = th.slot[a];
+                tw.c[a] = th.c[a];
+            }
+            float res[3];
+            load_mlp_residual(p, bd, th.mlp_s, xface1, y, z, res);
+            boundary_velocity<float>(reinterpret_cast<const float*>(p.ring), p.ring_slot_elems, bd, xface1, y, z, tw, ue);
+            add_mlp_residual<float>(p, bd, res, ue);
+        }
+        if (xface0) {
+            drho.x = th.drho_b;
+            ux.x = ue[0];
+            uy.x = ue[1];
+            uz.x = ue[2];
+        } else {
+            drho.y = th.drho_b;
+            ux.y = ue[0];
+            uy.y = ue[1];
+            uz.y = ue[2];
+        }
+    }
+}
+
 // Consumer thread c (0 .. 479) of one tile of 960 sites takes the adjacent
 // sites s0 + 2c and s0 + 2c + 1 (same row: E and s0 are even), so a warp
 // reads and writes 64 consecutive sites with one word per lane.  Same
@@ -578,40 +625,7 @@ __device__ __forceinline__ void staged_tile_pair(const SCParams& p, const Staged
 
     // boundary sites: equilibrium of the boundary velocity from the ring
     if (bnd0 || bnd1) {
-        if (brow) {  // a row on a y or z face (its x-face sites, which belong to the x faces, follow)
-            const int f = !py && y == 0 ? 2 : (!py && y == Ei - 1 ? 3 : (z == 0 ? 4 : 5));
-            float2 u[3];
-            boundary_velocity_pair(p, th, f, f < 4 ? z : y, x, u);
-            ux = u[0];
-            uy = u[1];
-            uz = u[2];
-            drho = f2(th.drho_b);
-        }
-        if (xface0 || xface1) {
-            if (!staged_edges) {
-                TimeWeights<float> tw;
-#pragma unroll
-                for (int a = 0; a < 4; a++) {
-                    tw.slot[a] = th.slot[a];
-                    tw.c[a] = th.c[a];
-                }
-                float res[3];
-                load_mlp_residual(p, bd, th.mlp_s, xface1, y, z, res);
-                boundary_velocity<float>(reinterpret_cast<const float*>(p.ring), p.ring_slot_elems, bd, xface1, y, z, tw, ue);
-                add_mlp_residual<float>(p, bd, res, ue);
-            }
-            if (xface0) {
-                drho.x = th.drho_b;
-                ux.x = ue[0];
-                uy.x = ue[1];
-                uz.x = ue[2];
-            } else {
-                drho.y = th.drho_b;
-                ux.y = ue[0];
-                uy.y = ue[1];
-                uz.y = ue[2];
-            }
-        }
+        boundary_pair(p, th, row, x, y, z, brow, xface0, xface1, staged_edges, ue, ux, uy, uz, drho);
         rho = add2(f2(1.f), drho);
     }
 
@@ -678,13 +692,12 @@ __device__ __forceinline__ void staged_tile_pair(const SCParams& p, const Staged
     }
 }
 
-// Consumer body of a box with the fluctuating collision (lbt_fluct.cuh): the
-// thread's sites (the adjacent pair s0 + 2c, s0 + 2c + 1 when SPT = 2, site
-// s0 + c when SPT = 1) pulled into registers, the stage released, then site by
-// site the moments and either the boundary equilibrium or the fluctuating
-// collision with the site's Philox noise of step n.  Boxes with a body force
-// or a chain do not take this path.
-template <int ST, int SPT, bool PER>
+// Consumer body of a box with the fluctuating collision (lbt_fluct.cuh), one
+// site a thread (FP64, and the reduced formats with one site a thread): the
+// site pulled into registers, the stage released, then the moments and either
+// the boundary equilibrium or the fluctuating collision with the site's Philox
+// noise of step n.  Boxes with a body force or a chain do not take this path.
+template <int ST, bool PER>
 __device__ __forceinline__ void staged_tile_fluct(const SCParams& p, const StagedTile<ST>& th,
                                                   const unsigned char* stage, uint64_t* empty, int64_t n)
 {
@@ -692,9 +705,9 @@ __device__ __forceinline__ void staged_tile_fluct(const SCParams& p, const Stage
     using E = typename S::E;
     using A = typename S::A;
     using R = typename S::R;
-    constexpr int H = Staged<ST, SPT>::kHalo;
+    constexpr int H = Staged<ST, 1>::kHalo;
     const int tid = threadIdx.x;
-    const int s0 = (int)th.s0;
+    const int s = (int)th.s0 + tid;
     const BoxDev& bd = th.bd;
     const int Ei = bd.E;
     const int n3 = (int)bd.n3;
@@ -702,92 +715,251 @@ __device__ __forceinline__ void staged_tile_fluct(const SCParams& p, const Stage
     const bool px = per & 1, py = per & 2, pz = per & 4;
     const E* Ab = reinterpret_cast<const E*>(p.A) + bd.f_off;
     E* Bb = reinterpret_cast<E*>(p.B) + bd.f_off;
-    auto local = [&](int k) { return SPT == 2 ? 2 * tid + k : tid; };
 
-    int xs_[SPT], ys_[SPT], zs_[SPT];
-    bool act[SPT], bnd[SPT];
-#pragma unroll
-    for (int k = 0; k < SPT; k++) {
-        const int s = s0 + local(k);
-        act[k] = s < n3;
-        const int sc = act[k] ? s : 0;
-        const int row = div_e(sc, bd.div_magic);
-        xs_[k] = sc - row * Ei;
-        zs_[k] = div_e(row, bd.div_magic);
-        ys_[k] = row - zs_[k] * Ei;
-        bnd[k] = act[k] && ((!px && (xs_[k] == 0 || xs_[k] == Ei - 1)) || (!py && (ys_[k] == 0 || ys_[k] == Ei - 1)) ||
-                            (!pz && (zs_[k] == 0 || zs_[k] == Ei - 1)));
-    }
-    A f[kQ][SPT];
+    const bool act = s < n3;
+    const int row = div_e(act ? s : 0, bd.div_magic);
+    const int x = (act ? s : 0) - row * Ei;
+    const int z = div_e(row, bd.div_magic);
+    const int y = row - z * Ei;
+    const bool bnd = act && ((!px && (x == 0 || x == Ei - 1)) || (!py && (y == 0 || y == Ei - 1)) ||
+                             (!pz && (z == 0 || z == Ei - 1)));
+    A d[kQ], r = A(0), j[3] = {A(0), A(0), A(0)};
 #pragma unroll
     for (int i = 0; i < kQ; i++) {
         const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
-        const E* row = reinterpret_cast<const E*>(stage + i * Staged<ST, SPT>::kRowStride);
-#pragma unroll
-        for (int k = 0; k < SPT; k++) {
-            A v = S::in(row[H + local(k) - cx]);
-            if (PER) {
-                const int xs = xs_[k] - cx, ys = ys_[k] - cy, zs = zs_[k] - cz;
-                const bool wrap = (px && (xs < 0 || xs >= Ei)) || (py && (ys < 0 || ys >= Ei)) ||
-                                  (pz && (zs < 0 || zs >= Ei));
-                if (wrap && act[k])
-                    v = S::in(Ab[(int64_t)i * n3 + ((int64_t)wrapi(zs, Ei) * Ei + wrapi(ys, Ei)) * Ei + wrapi(xs, Ei)]);
-            }
-            f[i][k] = (act[k] && !bnd[k]) ? v : A(0);
+        A v = S::in(reinterpret_cast<const E*>(stage + i * Staged<ST, 1>::kRowStride)[H + tid - cx]);
+        if (PER) {
+            const int xs = x - cx, ys = y - cy, zs = z - cz;
+            const bool wrap = (px && (xs < 0 || xs >= Ei)) || (py && (ys < 0 || ys >= Ei)) ||
+                              (pz && (zs < 0 || zs >= Ei));
+            if (wrap && act)
+                v = S::in(Ab[(int64_t)i * n3 + ((int64_t)wrapi(zs, Ei) * Ei + wrapi(ys, Ei)) * Ei + wrapi(xs, Ei)]);
         }
+        d[i] = act && !bnd ? v : A(0);
+        r += d[i];
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+            if (cvec(i, c)) j[c] += cvec(i, c) * d[i];
     }
     __syncwarp();
     if ((tid & 31) == 0) mbar_arrive(empty);  // this warp is done with the stage
 
-    const FluctDev& fd = p.fluct[th.box];
-    bool nonfinite = false;
+    const A rho = A(1) + r;
+    const bool nonfinite = !(rho > A(0) && rho < A(1e30));
+    A out[kQ];
+    if (bnd) {  // boundary equilibrium of the boundary velocity, as in the BGK bodies
+        TimeWeights<R> tw;
 #pragma unroll
-    for (int k = 0; k < SPT; k++) {
-        A d[kQ], r = A(0), jx = A(0), jy = A(0), jz = A(0);
-#pragma unroll
-        for (int i = 0; i < kQ; i++) {
-            d[i] = f[i][k];
-            r += d[i];
-            if (cvec(i, 0)) jx += cvec(i, 0) * d[i];
-            if (cvec(i, 1)) jy += cvec(i, 1) * d[i];
-            if (cvec(i, 2)) jz += cvec(i, 2) * d[i];
+        for (int a = 0; a < 4; a++) {
+            tw.slot[a] = th.slot[a];
+            tw.c[a] = th.c[a];
         }
-        const A rho = A(1) + r;
-        nonfinite |= !(rho > A(0) && rho < A(1e30));
-        A out[kQ];
-        if (bnd[k]) {  // boundary equilibrium of the boundary velocity, as in the BGK bodies
-            TimeWeights<R> tw;
+        int pp, qq;
+        const int fc = owning_face(x, y, z, Ei, per, pp, qq);
+        R ub[3];
+        boundary_velocity<R>(reinterpret_cast<const R*>(p.ring), p.ring_slot_elems, bd, fc, pp, qq, tw, ub);
+        const A dr = th.drho_b, rb = A(1) + dr;
+        const A u0 = (A)ub[0], u1 = (A)ub[1], u2 = (A)ub[2];
+        const A usq = A(1.5) * (u0 * u0 + u1 * u1 + u2 * u2);
 #pragma unroll
-            for (int a = 0; a < 4; a++) {
-                tw.slot[a] = th.slot[a];
-                tw.c[a] = th.c[a];
-            }
-            int pp, qq;
-            const int fc = owning_face(xs_[k], ys_[k], zs_[k], Ei, per, pp, qq);
-            R ub[3];
-            boundary_velocity<R>(reinterpret_cast<const R*>(p.ring), p.ring_slot_elems, bd, fc, pp, qq, tw, ub);
-            const A dr = th.drho_b, rb = A(1) + dr;
-            const A u0 = (A)ub[0], u1 = (A)ub[1], u2 = (A)ub[2];
-            const A usq = A(1.5) * (u0 * u0 + u1 * u1 + u2 * u2);
+        for (int i = 0; i < kQ; i++) out[i] = fluct_deq<A>(i, dr, rb, u0, u1, u2, usq);
+    } else {
+        const A inv = A(1) / rho;
+        fluct_collide<A>(d, r, j[0] * inv, j[1] * inv, j[2] * inv, p.fluct[th.box], n, s, out);
+    }
+    if (act)
 #pragma unroll
-            for (int i = 0; i < kQ; i++) {
-                A cu = A(0);
-                if (cvec(i, 0)) cu += cvec(i, 0) * u0;
-                if (cvec(i, 1)) cu += cvec(i, 1) * u1;
-                if (cvec(i, 2)) cu += cvec(i, 2) * u2;
-                out[i] = wgt<A>(i) * (dr + rb * (A(3) * cu + A(4.5) * cu * cu - usq));
+        for (int i = 0; i < kQ; i++) Bb[(int64_t)i * n3 + s] = S::out(out[i]);
+    if (__any_sync(0xffffffffu, nonfinite) && (tid & 31) == 0) atomicCAS(&p.status[th.box], 0, LB_ERR_NONFINITE);
+}
+
+// The fluctuating collision of two adjacent sites per thread (FP32 and 16-bit
+// storage), in packed FP32.  An even mode sees only the sum of an opposite pair
+// of populations, an odd one only the difference, so the two transforms come
+// down to about a hundred additions for both sites together; the relaxation
+// factors and noise amplitudes are read in FP32, folded with the mode norms.
+// Arithmetic bound (the transforms, eight Philox calls a thread): 96^3 FP32 in
+// 53.9 us a step; with 19 x 15 scalar transforms a site, the parameters
+// converted from FP64 for every site and four-byte stores two sites apart, 109.
+template <int ST, bool PER>
+__device__ __forceinline__ void staged_tile_fluct_pair(const SCParams& p, const StagedTile<ST>& th,
+                                                       const unsigned char* stage, uint64_t* empty, int64_t n)
+{
+    static_assert(ST != kF64, "the paired body works in FP32");
+    using S = Stor<ST>;
+    using E = typename S::E;
+    using IO = PairIO<ST>;
+    constexpr int H = Staged<ST, 2>::kHalo;
+    const int tid = threadIdx.x;
+    const BoxDev& bd = th.bd;
+    const int Ei = bd.E;
+    const int n3 = (int)bd.n3;
+    const int per = bd.per_mask;
+    const bool px = per & 1, py = per & 2, pz = per & 4;
+    const E* Ab = reinterpret_cast<const E*>(p.A) + bd.f_off;
+    const int s = (int)th.s0 + 2 * tid;  // first site of the pair (even)
+    const bool act = s < n3;             // n3 is even: both sites or none
+    const int row = div_e(act ? s : 0, bd.div_magic);
+    const int x = (act ? s : 0) - row * Ei;
+    const int z = div_e(row, bd.div_magic);
+    const int y = row - z * Ei;
+    const bool brow = act && ((!py && (y == 0 || y == Ei - 1)) || (!pz && (z == 0 || z == Ei - 1)));
+    const bool xface0 = act && !px && x == 0, xface1 = act && !px && x + 1 == Ei - 1;
+    const bool bnd0 = brow || xface0, bnd1 = brow || xface1;
+
+    float2 f[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; i++) {
+        const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
+        const E* src = reinterpret_cast<const E*>(stage + i * Staged<ST, 2>::kRowStride);
+        float2 v = cx == 0 ? IO::even(src, H + 2 * tid) : IO::any(src, H + 2 * tid - cx);
+        if (PER) {
+            const int ys = y - cy, zs = z - cz;
+            const bool wyz = (py && (ys < 0 || ys >= Ei)) || (pz && (zs < 0 || zs >= Ei));
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const int xs = x + k - cx;
+                if ((wyz || (px && (xs < 0 || xs >= Ei))) && act) {
+                    const float w = S::in(
+                        Ab[(int64_t)i * n3 + ((int64_t)wrapi(zs, Ei) * Ei + wrapi(ys, Ei)) * Ei + wrapi(xs, Ei)]);
+                    if (k == 0) v.x = w;
+                    else v.y = w;
+                }
             }
-        } else {
-            const A inv = A(1) / rho;
-            fluct_collide<A>(d, r, jx * inv, jy * inv, jz * inv, fd, n, s0 + local(k), out);
         }
-        if (act[k]) {
-            E* o = Bb + s0 + local(k);
+        f[i] = v;  // boundary lanes: finite, multiplied by zero below
+    }
+    __syncwarp();
+    if ((tid & 31) == 0) mbar_arrive(empty);  // this warp is done with the stage
+
+    // opposite pairs: sums in f[i], differences in f[i + 1] (i odd)
+    float2 r = f[0], j[3];
 #pragma unroll
-            for (int i = 0; i < kQ; i++) o[(int64_t)i * n3] = S::out(out[i]);
+    for (int i = 1; i < kQ; i += 2) {
+        const float2 a = f[i], b = f[i + 1];
+        f[i] = add2(a, b);
+        f[i + 1] = sub2(a, b);
+        r = add2(r, f[i]);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            if (i == 1 + 2 * c) j[c] = f[i + 1];  // the axis pairs come first
+            else if (cvec(i, c) > 0) j[c] = add2(j[c], f[i + 1]);
+            else if (cvec(i, c) < 0) j[c] = sub2(j[c], f[i + 1]);
         }
     }
+    float2 rho = add2(f2(1.f), r);
+    const bool nonfinite = (act && !bnd0 && !(rho.x > 0.f && rho.x < 1e30f)) || (act && !bnd1 && !(rho.y > 0.f && rho.y < 1e30f));
     if (__any_sync(0xffffffffu, nonfinite) && (tid & 31) == 0) atomicCAS(&p.status[th.box], 0, LB_ERR_NONFINITE);
+    // 1 / rho to half an ulp (one Newton step on the hardware's approximation):
+    // its error goes straight into the momentum the equilibrium carries
+    float2 inv = make_float2(fast_inverse(rho.x), fast_inverse(rho.y));
+    inv = fma2(inv, fma2(mul2(f2(-1.f), rho), inv, f2(1.f)), inv);
+    float2 ux = mul2(j[0], inv), uy = mul2(j[1], inv), uz = mul2(j[2], inv), drho = r;
+    const float2 srho = make_float2(sqrtf(rho.x), sqrtf(rho.y));
+    if (bnd0 || bnd1) {
+        float ue[3];
+        boundary_pair(p, th, row, x, y, z, brow, xface0, xface1, false, ue, ux, uy, uz, drho);
+        rho = add2(f2(1.f), drho);
+    }
+    // equilibrium of a pair: even part q cu^2 + b, odd part t cu
+    const float2 xx = mul2(ux, ux), yy = mul2(uy, uy), zz = mul2(uz, uz);
+    const float2 base = fma2(rho, mul2(f2(-1.5f), add2(xx, add2(yy, zz))), drho);
+    // (the FP32 value of 1/18 is 7e-9 off, that of 1/6 3e-8: the momentum a step
+    // carries over would grow by as much every step)
+    const float2 k18 = mul2(f2(1.f / 18.f), rho);
+    const float2 b18 = mul2(f2(1.f / 18.f), base), b36 = mul2(f2(0.5f), b18);
+    const float2 q18 = mul2(f2(4.5f), k18), q36 = mul2(f2(2.25f), k18);
+    const float2 t18 = mul2(f2(3.f), k18), t36 = mul2(f2(1.5f), k18);
+    auto equilibrium = [&](int i, float2& even, float2& odd) {
+        const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
+        const bool axis = i < 7;
+        const float2 first = cx ? ux : (cy ? uy : uz), second = cz ? uz : uy;
+        const float2 cu = axis ? first : ((cx ? (cy ? cy : cz) : cz) > 0 ? add2(first, second) : sub2(first, second));
+        even = fma2(axis ? q18 : q36, axis ? (cx ? xx : (cy ? yy : zz)) : mul2(cu, cu), axis ? b18 : b36);
+        odd = mul2(axis ? t18 : t36, cu);
+    };
+    // non-equilibrium sums and differences, then the moments of modes 4 .. 18 (lbt_fluct.cuh)
+    const float2 n0 = fma2(f2(-6.f), b18, f[0]);
+#pragma unroll
+    for (int i = 1; i < kQ; i += 2) {
+        float2 even, odd;
+        equilibrium(i, even, odd);
+        f[i] = fma2(f2(-2.f), even, f[i]);
+        f[i + 1] = fma2(f2(-2.f), odd, f[i + 1]);
+    }
+    float2 m[15];
+    {
+        const float2 exy = add2(f[7], f[9]), exz = add2(f[11], f[13]), eyz = add2(f[15], f[17]);
+        const float2 es = add2(add2(exy, exz), eyz), as = add2(add2(f[1], f[3]), f[5]);
+        m[0] = sub2(es, n0);
+        m[12] = add2(fma2(f2(-2.f), as, es), n0);
+        const float2 ax = fma2(f2(3.f), f[1], mul2(f2(-1.f), as)), ex = fma2(f2(-3.f), eyz, es);
+        m[1] = add2(ax, ex);
+        m[13] = sub2(ex, ax);
+        const float2 ay = sub2(f[3], f[5]), ey = sub2(exy, exz);
+        m[2] = add2(ay, ey);
+        m[14] = sub2(ey, ay);
+        m[3] = sub2(f[7], f[9]);
+        m[4] = sub2(f[15], f[17]);
+        m[5] = sub2(f[11], f[13]);
+        const float2 sx = add2(f[8], f[10]), tx = add2(f[12], f[14]);
+        m[6] = fma2(f2(-2.f), f[2], add2(sx, tx));
+        m[9] = sub2(sx, tx);
+        const float2 sy = sub2(f[8], f[10]), ty = add2(f[16], f[18]);
+        m[7] = fma2(f2(-2.f), f[4], add2(sy, ty));
+        m[10] = sub2(ty, sy);
+        const float2 sz = sub2(f[12], f[14]), tz = sub2(f[16], f[18]);
+        m[8] = fma2(f2(-2.f), f[6], add2(sz, tz));
+        m[11] = sub2(sz, tz);
+    }
+    // relaxed moments plus noise, over their norms; none on boundary sites
+    const float2 keep = make_float2(bnd0 ? 0.f : 1.f, bnd1 ? 0.f : 1.f);
+    const FluctDev& fd = p.fluct[th.box];
+    const uint32_t k0 = (uint32_t)fd.seed, k1 = (uint32_t)(fd.seed >> 32);
+#pragma unroll
+    for (int blk = 0; blk < 4; blk++) {
+        uint32_t xa[4] = {(uint32_t)n, (uint32_t)s, (uint32_t)blk, 0xF1u}, xb[4] = {(uint32_t)n, (uint32_t)s + 1, (uint32_t)blk, 0xF1u};
+        philox4x32_10(xa, k0, k1);
+        philox4x32_10(xb, k0, k1);
+        const float4 g = __ldg(reinterpret_cast<const float4*>(fd.gamma_f) + blk);
+        const float4 a = __ldg(reinterpret_cast<const float4*>(fd.amp_f) + blk);
+        const float gk[4] = {g.x, g.y, g.z, g.w}, ak[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int w = 0; w < 4; w++)
+            if (4 * blk + w < 15) {
+                const float2 xi = make_float2(unit_uniform_t<float>(xa[w]), unit_uniform_t<float>(xb[w]));
+                float2& mk = m[4 * blk + w];
+                mk = mul2(keep, fma2(f2(gk[w]), mk, mul2(mul2(f2(ak[w]), srho), xi)));
+            }
+    }
+    // back to the populations: equilibrium + w (even part +- odd part)
+    E* out = reinterpret_cast<E*>(p.B) + bd.f_off + s;
+    if (act) IO::store(out, fma2(f2(6.f), b18, mul2(f2(1.f / 3.f), sub2(m[12], m[0]))));
+    const float2 G = add2(m[0], m[12]), Hh = add2(m[1], m[13]), I = add2(m[2], m[14]);
+    const float2 h = sub2(m[1], m[13]), v = sub2(m[2], m[14]), c2 = mul2(f2(-2.f), m[12]);
+#pragma unroll
+    for (int i = 1; i < kQ; i += 2) {
+        out += i == 1 ? n3 : 2 * n3;  // row of population i; population i + 1 is one row further
+        float2 even, odd, e, o;
+        equilibrium(i, even, odd);
+        if (i == 1) e = fma2(f2(2.f), h, c2);
+        else if (i == 3) e = add2(sub2(v, h), c2);
+        else if (i == 5) e = sub2(sub2(c2, h), v);
+        else if (i < 11) e = i == 7 ? add2(add2(add2(G, Hh), I), m[3]) : sub2(add2(add2(G, Hh), I), m[3]);
+        else if (i < 15) e = i == 11 ? add2(sub2(add2(G, Hh), I), m[5]) : sub2(sub2(add2(G, Hh), I), m[5]);
+        else e = i == 15 ? add2(fma2(f2(-2.f), Hh, G), m[4]) : sub2(fma2(f2(-2.f), Hh, G), m[4]);
+        if (i < 7) o = mul2(f2(-2.f), m[6 + i / 2]);
+        else if (i < 11) o = i == 7 ? add2(add2(m[6], m[9]), sub2(m[7], m[10])) : sub2(add2(m[6], m[9]), sub2(m[7], m[10]));
+        else if (i < 15) o = i == 11 ? add2(sub2(m[6], m[9]), add2(m[8], m[11])) : sub2(sub2(m[6], m[9]), add2(m[8], m[11]));
+        else o = i == 15 ? add2(add2(m[7], m[10]), sub2(m[8], m[11])) : sub2(add2(m[7], m[10]), sub2(m[8], m[11]));
+        const float2 w = f2(i < 7 ? 1.f / 18.f : 1.f / 36.f);
+        even = fma2(w, e, even);
+        odd = fma2(w, o, odd);
+        if (act) {
+            IO::store(out, add2(even, odd));
+            IO::store(out + n3, sub2(even, odd));
+        }
+    }
 }
 
 // Consumer warps: take the stages in order until the producer posts the end.
@@ -832,8 +1004,13 @@ __device__ __forceinline__ void staged_consume(const SCParams& p, unsigned char*
                     for (int i = 0; i < kQ; i++) Bb[(int64_t)i * bd.n3 + s0 + t] = Ab[(int64_t)i * bd.n3 + s0 + t];
         } else if (KIND == 2 && bd.fluct) {
             if constexpr (KIND == 2) {
-                if (bd.per_mask) staged_tile_fluct<ST, SPT, true>(p, th, stage, &hd->empty[st], n);
-                else staged_tile_fluct<ST, SPT, false>(p, th, stage, &hd->empty[st], n);
+                if constexpr (SPT == 2 && ST != kF64) {
+                    if (bd.per_mask) staged_tile_fluct_pair<ST, true>(p, th, stage, &hd->empty[st], n);
+                    else staged_tile_fluct_pair<ST, false>(p, th, stage, &hd->empty[st], n);
+                } else {
+                    if (bd.per_mask) staged_tile_fluct<ST, true>(p, th, stage, &hd->empty[st], n);
+                    else staged_tile_fluct<ST, false>(p, th, stage, &hd->empty[st], n);
+                }
             }
         } else if constexpr (SPT == 2 && ST != kF64) {  // adjacent site pairs, packed FP32
             if (!GENERAL) {
