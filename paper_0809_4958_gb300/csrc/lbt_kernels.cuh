@@ -1744,6 +1744,10 @@ __global__ void __launch_bounds__(kFieldsThreads) k_fields(const typename Stor<S
     const int Ei = bd.E, per = bd.per_mask, gpr = Ei / VW, fe = Ei * Ei;
     const bool px = per & 1, py = per & 2, pz = per & 4;
     const int n3 = (int)bd.n3, lane = threadIdx.x & 31;
+    // A read-out of many boxes is many small launches: each is a programmatic
+    // dependent of the one before and lets the next be scheduled at once
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int G = blockIdx.x * kFieldsThreads + threadIdx.x; G < n3 / VW; G += gridDim.x * kFieldsThreads) {
         const int row = G / gpr, xg = G - row * gpr;
         const int z = row / Ei, y = row - z * Ei;
@@ -1968,13 +1972,7 @@ cudaError_t launch_staged(const SCParams& p, int ctas, cudaStream_t s)
     static int attr_done[kMaxDevices] = {};  // per instantiation and device
     cudaError_t e = smem_attr_per_device(k_stream_collide_staged<ST, SPT, KIND>, G::kSmemBytes, attr_done);
     if (e != cudaSuccess) return e;
-    int sms = 0;
-    if (ctas <= 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
-    int64_t grid = ctas > 0 ? ctas : sms;
+    int64_t grid = ctas;  // the persistent grid (the caller's: one block per SM by default)
     if (grid > p.total_tiles) grid = p.total_tiles;
     if (grid < 1) return cudaSuccess;
     // programmatic dependent launch: the blocks may be scheduled before the
@@ -2116,11 +2114,18 @@ cudaError_t launch_fields(const void* A, const BoxDev& bd, int what, void* dst, 
     const typename Stor<ST>::E* a = reinterpret_cast<const typename Stor<ST>::E*>(A);
     const int grid = grid_for(bd.n3 / VW, kFieldsThreads, 1 << 20);
     const int vec = reinterpret_cast<uintptr_t>(dst) % 16 == 0;  // the caller's buffer may start anywhere
-    if (what == 0)
-        k_fields<ST, VW, 0><<<grid, kFieldsThreads, 0, s>>>(a, bd, reinterpret_cast<R*>(dst), vec);
-    else
-        k_fields<ST, VW, 1><<<grid, kFieldsThreads, 0, s>>>(a, bd, reinterpret_cast<R*>(dst), vec);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kFieldsThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    R* d = reinterpret_cast<R*>(dst);
+    return what == 0 ? cudaLaunchKernelEx(&cfg, k_fields<ST, VW, 0>, a, bd, d, vec)
+                     : cudaLaunchKernelEx(&cfg, k_fields<ST, VW, 1>, a, bd, d, vec);
 }
 
 template <int ST>

@@ -187,6 +187,7 @@ struct StagedTile {
     using R = typename Stor<ST>::R;
     BoxDev bd;
     int64_t s0;
+    int64_t step;  // the step n -> n + 1 of the launch
     int32_t box;
     int32_t mlp_s;
     int32_t frozen;  // the box carries an error status: its state does not change
@@ -967,8 +968,7 @@ __device__ __forceinline__ void staged_tile_fluct_pair(const SCParams& p, const 
 // that tile body is compiled in (fewer registers than the kernel that carries
 // all bodies).
 template <int ST, int SPT, int KIND>
-__device__ __forceinline__ void staged_consume(const SCParams& p, unsigned char* smem, StagedHeader<ST>* hd,
-                                               int64_t n)
+__device__ __forceinline__ void staged_consume(const SCParams& p, unsigned char* smem, StagedHeader<ST>* hd)
 {
     constexpr bool GENERAL = KIND > 0;
     using G = Staged<ST, SPT>;
@@ -1005,11 +1005,11 @@ __device__ __forceinline__ void staged_consume(const SCParams& p, unsigned char*
         } else if (KIND == 2 && bd.fluct) {
             if constexpr (KIND == 2) {
                 if constexpr (SPT == 2 && ST != kF64) {
-                    if (bd.per_mask) staged_tile_fluct_pair<ST, true>(p, th, stage, &hd->empty[st], n);
-                    else staged_tile_fluct_pair<ST, false>(p, th, stage, &hd->empty[st], n);
+                    if (bd.per_mask) staged_tile_fluct_pair<ST, true>(p, th, stage, &hd->empty[st], th.step);
+                    else staged_tile_fluct_pair<ST, false>(p, th, stage, &hd->empty[st], th.step);
                 } else {
-                    if (bd.per_mask) staged_tile_fluct<ST, true>(p, th, stage, &hd->empty[st], n);
-                    else staged_tile_fluct<ST, false>(p, th, stage, &hd->empty[st], n);
+                    if (bd.per_mask) staged_tile_fluct<ST, true>(p, th, stage, &hd->empty[st], th.step);
+                    else staged_tile_fluct<ST, false>(p, th, stage, &hd->empty[st], th.step);
                 }
             }
         } else if constexpr (SPT == 2 && ST != kF64) {  // adjacent site pairs, packed FP32
@@ -1135,7 +1135,7 @@ __device__ __forceinline__ const float* edge_runs(const SCParams& p, StagedTile<
 // under a body force 71.6 and 58.7; one more round trip a tile made them 330
 // and 83.)
 template <int ST, int SPT, int KIND>
-__device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char* smem, StagedHeader<ST>* hd, int64_t n)
+__device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char* smem, StagedHeader<ST>* hd)
 {
     using G = Staged<ST, SPT>;
     using E = typename Stor<ST>::E;
@@ -1157,10 +1157,20 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
     const uint64_t pol = p.hint_loads ? l2_evict_first_policy() : 0;
     unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p.tile_counter);
     const int run = p.claim;  // neighbouring tiles of one claim
-    const bool back = (n & 1) && p.withhold_tile < 0;
-    long long next = lane == 0 ? (long long)atomicAdd(ctr, (unsigned long long)run) : 0;
-    next = __shfl_sync(0xffffffffu, next, 0);
+    // the first claim of a block is fixed, the counter deals out the rest
+    const long long dealt = (long long)gridDim.x * run;
+    long long next = (long long)blockIdx.x * run;
     int left = run;  // tiles of the claim not yet taken
+    // the record of an only box (written by nothing but copies between launches)
+    const bool only = p.nboxes == 1;
+    uint64_t only_word = 0;
+    if (only && lane < (int)(sizeof(BoxDev) / 8)) only_word = reinterpret_cast<const uint64_t*>(p.boxes)[lane];
+    // Launched as a programmatic dependent of the kernel before it on the
+    // stream (the previous step's last): everything up to here may run while
+    // that kernel does.  Wait for it to complete and its writes to be visible.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int64_t n = *p.step;
+    const bool back = (n & 1) && p.withhold_tile < 0;
     // of the current box
     int64_t tile_lo = 0, tile_hi = 0;  // its tiles
     uint64_t hw[kMine];
@@ -1197,14 +1207,15 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
             return;
         }
         long long claimed = 0;
-        if (left == 1 && lane == 0) claimed = (long long)atomicAdd(ctr, (unsigned long long)run);  // overlaps this tile's copies
+        if (left == 1 && lane == 0)
+            claimed = dealt + (long long)atomicAdd(ctr, (unsigned long long)run);  // overlaps this tile's copies
         if (t < tile_lo || t >= tile_hi) {  // another box: its record and what the collision and the boundary need at this step
             const int b = locate_box_warp(p, t, lane);
-            const BoxDev& bd = p.boxes[b];
-            tile_lo = p.tile_prefix[b];
-            tile_hi = p.tile_prefix[b + 1];
+            tile_lo = only ? 0 : p.tile_prefix[b];
+            tile_hi = only ? p.total_tiles : p.tile_prefix[b + 1];
             if (lane < (int)(sizeof(BoxDev) / 8))
-                reinterpret_cast<uint64_t*>(&th.bd)[lane] = reinterpret_cast<const uint64_t*>(&bd)[lane];
+                reinterpret_cast<uint64_t*>(&th.bd)[lane] =
+                    only ? only_word : reinterpret_cast<const uint64_t*>(p.boxes + b)[lane];
             const int frozen = p.status[b] != 0;
             __syncwarp();
             if (lane == 0) {
@@ -1216,6 +1227,7 @@ __device__ __forceinline__ void staged_produce(const SCParams& p, unsigned char*
                     frame_accel_at(th.bd, p.faccel, p.ring_slots, n, a);
                     for (int c = 0; c < 3; c++) th.bd.accel[c] = a[c];
                 }
+                th.step = n;
                 th.box = b;
                 th.frozen = frozen;
                 for (int a = 0; a < 4; a++) {
@@ -1330,30 +1342,26 @@ __global__ void __launch_bounds__(kStagedThreads, 1) k_stream_collide_staged(SCP
         }
         fence_mbar_init();
     }
-    // Launched as a programmatic dependent of the kernel before it on the
-    // stream (the previous step's last): the block may start while that kernel
-    // runs, and everything above touched only shared memory.  Wait here for it
-    // to complete and its writes to be visible.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int64_t n = *p.step;
-    __syncthreads();  // the barriers are initialised, and every thread has read the step
+    __syncthreads();
     if (threadIdx.x >= kStagedConsumers) {
-        staged_produce<ST, SPT, KIND>(p, smem, hd, n);  // the whole last warp
+        staged_produce<ST, SPT, KIND>(p, smem, hd);  // the whole last warp
         // Without chains no forced re-collision follows: the last block to run
-        // out of tiles ends the step (no claim and no reading of the step is
-        // left then; a producer that gave up counts as well).
+        // out of tiles ends the step (only producers claim tiles or read the
+        // step, and all are done then; a producer that gave up counts as well).
         if (p.ends_step && (threadIdx.x & 31) == 0) {
             unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p.tile_counter);
             __threadfence();
             if (atomicAdd(ctr + 1, 1ull) == gridDim.x - 1) {
                 ctr[0] = 0;
                 ctr[1] = 0;
-                *const_cast<int64_t*>(p.step) = n + 1;
+                *const_cast<int64_t*>(p.step) += 1;
             }
         }
         return;
     }
-    staged_consume<ST, SPT, KIND>(p, smem, hd, n);
+    // the consumers' own reads of global memory also come after the kernel before
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    staged_consume<ST, SPT, KIND>(p, smem, hd);
 }
 
 }  // namespace lbt
