@@ -844,10 +844,13 @@ __device__ __noinline__ int rebuild_chain_list(const typename Vec4<MT>::T* X, un
 // start positions and rebuilt by the MD threads after a flagged barrier.
 // Symplectic Euler as in md_substeps.  Called by every thread of the block;
 // returns an error code (0 = none), the same in all threads.
-template <class MT>
+//
+// idle(first, count): called once by the warps that take no part in the
+// substeps, with their thread index among themselves and their number.
+template <class MT, class Idle>
 __device__ __forceinline__ int md_chain_pairs(const BeadParams& p, const ChainDev& ch, int N, int64_t n, int b,
                                               MT* sXbuf, MT (*sU)[3], MT (*sV)[3], double (*sR)[3], MT (*sP)[3],
-                                              unsigned char (*sNb)[kMaxTasks], int* sErrP)
+                                              unsigned char (*sNb)[kMaxTasks], int* sErrP, const Idle& idle)
 {
     using V4 = typename Vec4<MT>::T;
     __shared__ int sNbN[kMaxBeads];  // listed partners of each bead
@@ -963,17 +966,25 @@ __device__ __forceinline__ int md_chain_pairs(const BeadParams& p, const ChainDe
                 const int sub = c0 + sb;
                 const V4* Xc = sX4 + (sub & 1) * maxb;
                 V4* Xn = sX4 + ((sub + 1) & 1) * maxb;
-                // the lane's two fixed partners and its first two list slots
-                // in one branch-free block, so that the four pair
-                // computations interleave (empty slots are masked)
+                // the lane's two fixed partners and the list slots some lane of
+                // the warp uses, at most two, in one branch-free block, so that
+                // the pair computations interleave (a lane's empty slots are masked)
                 const V4 xi = namp > MT(0) ? sXi[sb * N + gg] : V4{};
-                const V4 ql = Xc[il], qr = Xc[ir], q0 = Xc[li & 255u], q1 = Xc[(li >> 8) & 255u];
                 const MT X[3] = {x0[0] + d[0], x0[1] + d[1], x0[2] + d[2]};
                 MT F[3] = {fx[0], fx[1], fx[2]}, G[3] = {MT(0), MT(0), MT(0)};
-                bool stretched = chain_pair<MT>(X, ql, fene, onl, pc, wca, F);
-                stretched |= chain_pair<MT>(X, qr, fene, onr, pc, wca, G);
-                chain_pair<MT>(X, q0, false, wca && 0 < mine, pc, wca, F);
-                chain_pair<MT>(X, q1, false, wca && 1 < mine, pc, wca, G);
+                bool stretched = false;
+                auto forces = [&](auto slots) {
+                    constexpr int kSlots = decltype(slots)::value;
+                    const V4 ql = Xc[il], qr = Xc[ir];
+                    const V4 q0 = kSlots > 0 ? Xc[li & 255u] : V4{}, q1 = kSlots > 1 ? Xc[(li >> 8) & 255u] : V4{};
+                    stretched = chain_pair<MT>(X, ql, fene, onl, pc, wca, F);
+                    stretched |= chain_pair<MT>(X, qr, fene, onr, pc, wca, G);
+                    if (kSlots > 0) chain_pair<MT>(X, q0, false, wca && 0 < mine, pc, wca, F);
+                    if (kSlots > 1) chain_pair<MT>(X, q1, false, wca && 1 < mine, pc, wca, G);
+                };
+                if (kmax > 1) forces(std::integral_constant<int, 2>{});
+                else if (kmax == 1) forces(std::integral_constant<int, 1>{});
+                else forces(std::integral_constant<int, 0>{});
 #pragma unroll
                 for (int a = 0; a < 3; a++) F[a] += G[a];
                 // the rest of the list (rare: a bead with more than four
@@ -1021,6 +1032,8 @@ __device__ __forceinline__ int md_chain_pairs(const BeadParams& p, const ChainDe
                     pack();
                 }
             }
+        } else if (c0 == 0) {
+            idle(tid - nmd, nthr - nmd);
         }
         __syncthreads();
         if (sErrP[0] || sErrP[1]) break;
@@ -1055,9 +1068,11 @@ __device__ __forceinline__ int md_chain_pairs(const BeadParams& p, const ChainDe
 // and divisions: 298 and 371; ROLES_US.)  Flags and errors as in md_chain_pairs.
 constexpr int kRoleBeads = kBeadThreadsMax / 4;  // beads the four roles' warps cover
 
+template <class Idle>
 __device__ __forceinline__ int md_chain_roles(const BeadParams& p, const ChainDev& ch, int N, int64_t n, int b,
                                               double* sXbuf, double (*sU)[3], double (*sV)[3], double (*sR)[3],
-                                              double (*sP)[3], unsigned char (*sNb)[kMaxTasks], int* sErrP)
+                                              double (*sP)[3], unsigned char (*sNb)[kMaxTasks], int* sErrP,
+                                              const Idle& idle)
 {
     using V4 = typename Vec4<double>::T;
     __shared__ int sNbN[kRoleBeads];  // listed partners of each bead
@@ -1243,6 +1258,8 @@ __device__ __forceinline__ int md_chain_roles(const BeadParams& p, const ChainDe
                     dref = d;
                 }
             }
+        } else if (c0 == 0) {
+            idle(tid - nmd, nthr - nmd);
         }
         __syncthreads();
         if (sErrP[0] || sErrP[1]) break;
@@ -1384,94 +1401,16 @@ __global__ void __launch_bounds__(kBeadThreadsMax) k_bead_couple(BeadParams p)
     }
     __syncthreads();
 
-    // 3. MD substeps (md_substeps below)
-    {
-        __shared__ int sErrP[2];
-        int err = 0;
-        if (p.beads_per_thread == 0) {
-            bool roles = false;
-            if constexpr (sizeof(MT) == 8) {
-                roles = N <= kRoleBeads && nthr >= 128 * ((N + 31) / 32);
-                if (roles) err = md_chain_roles(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
-            }
-            if (!roles) err = md_chain_pairs<MT>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
-        } else if (p.beads_per_thread == 1 && p.lanes == 8)
-            err = md_substeps_split<MT, 8>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
-        else if (p.beads_per_thread == 1 && p.lanes == 4)
-            err = md_substeps_split<MT, 4>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
-        else if (p.beads_per_thread == 2)
-            err = md_substeps<MT, 2>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
-        else
-            err = md_substeps<MT, 1>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
-        if (err) {
-            if (tid == 0) set_status(&p.status[b], err);
-            return;
-        }
-    }
-
-    // 4. centre of mass pinned at the box centre (one thread per bead; only
-    //    the warps holding beads reduce).  The sums run in MT over the offsets
-    //    from bead 0's start-of-step position, which are small: FP64 is slow
-    //    on this part, and the pin is re-applied every step, so the FP32
-    //    rounding of one step's shift does not accumulate.
-    double R[3] = {0, 0, 0};
-    MT V[3] = {0, 0, 0};
-    if (tid < N)
-        for (int a = 0; a < 3; a++) {
-            R[a] = sR[tid][a];
-            V[a] = sV[tid][a];
-        }
-    if (ch.pin_com >= 1) {
-        const int warp = tid >> 5, lane = tid & 31, nbw = (N + 31) >> 5;
-        if (warp < nbw)
-            for (int pass = 0; pass < 2; pass++) {
-                MT s[3];
-                for (int a = 0; a < 3; a++) {
-                    s[a] = tid < N ? (pass == 0 ? (MT)(R[a] - sRc[a]) : V[a]) : MT(0);
-                    for (int o = 16; o > 0; o >>= 1) s[a] += __shfl_xor_sync(0xffffffffu, s[a], o);
-                }
-                if (lane == 0)
-                    for (int a = 0; a < 3; a++) sRed[pass][warp][a] = s[a];
-            }
-        __syncthreads();
-        if (tid < N) {
-            MT com[3] = {0, 0, 0}, vcm[3] = {0, 0, 0};
-            for (int w = 0; w < nbw; w++)
-                for (int a = 0; a < 3; a++) {
-                    com[a] += sRed[0][w][a];
-                    vcm[a] += sRed[1][w][a];
-                }
-            const double centre = 0.5 * (Ei - 1);
-            const MT inv_n = sizeof(MT) == 8 ? (MT)ch.md_d[kMdInvN] : (MT)ch.md_f[kMdInvN];
-            for (int a = 0; a < 3; a++) {
-                R[a] += (centre - sRc[a]) - (double)(com[a] * inv_n);
-                if (ch.pin_com >= 2) V[a] = V[a] - vcm[a] * inv_n;
-            }
-        }
-    }
-    if (tid < N)
-        for (int a = 0; a < 3; a++) {
-            pos[3 * tid + a] = R[a];
-            vel[3 * tid + a] = (double)V[a];
-        }
-    if (p.hist_slots > 0 && tid < N) {  // the trajectory ring: positions after step n + 1
-        double* h = p.hist + ((n + 1) % p.hist_slots) * p.hist_stride + 3 * (int64_t)ch.bead_off;
-        for (int a = 0; a < 3; a++) h[3 * tid + a] = R[a];
-    }
-
-    // 5. force density at the stencil sites: every entry sums, in bead order,
-    //    the contributions of all beads whose stencil holds its site; entries
-    //    whose site an earlier bead already holds are marked duplicates.
-    //    Only beads whose stencil corner lies within one cell of this bead's on
-    //    every axis can share a site: each bead first lists those (in bead
-    //    order, itself included), then each entry scans its bead's list only.
-    ForceEntry* fl = p.forces + ch.force_off;
-    //    Eight threads per bead scan consecutive eighths of the chain and
-    //    merge their finds in order by a prefix sum over the eight.
-    {
+    // Beads whose stencils may share a site: only those whose stencil corner
+    // lies within one cell of a bead's on every axis, listed in bead order,
+    // itself included.  Eight threads per bead scan consecutive eighths of the
+    // chain and merge their finds in order by a prefix sum over the eight.  It
+    // needs the start-of-step stencils only, so that warps the substeps leave
+    // idle do it meanwhile (t, nt: thread among nt, whole warps).
+    auto near_lists = [&](int t, int nt) {
         const int part = (N + 7) >> 3;  // <= 32 beads per thread
-        for (int base = 0; base < 8 * N; base += nthr) {
-            const int e = base + tid;
+        for (int base = 0; base < 8 * N; base += nt) {
+            const int e = base + t;
             const bool act = e < 8 * N;
             const int bb = act ? e >> 3 : 0, r = e & 7;
             const int lo = r * part, hi = min(N, lo + part);
@@ -1503,9 +1442,103 @@ __global__ void __launch_bounds__(kBeadThreadsMax) k_bead_couple(BeadParams p)
                 if (r == 7) sStN[bb] = total <= kMaxStencilNb ? total : -1;  // -1: too many, scan every bead
             }
         }
+    };
+    // 3. MD substeps (md_substeps below)
+    bool listed = false;  // near_lists done by idle warps
+    {
+        __shared__ int sErrP[2];
+        int err = 0;
+        if (p.beads_per_thread == 0) {
+            const bool roles = sizeof(MT) == 8 && N <= kRoleBeads && nthr >= 128 * ((N + 31) / 32);
+            listed = nthr - (roles ? 128 * ((N + 31) / 32) : (2 * N + 31) & ~31) >= 64;
+            auto idle = [&](int t, int nt) {
+                if (listed) near_lists(t, nt);
+            };
+            if constexpr (sizeof(MT) == 8)
+                if (roles) err = md_chain_roles(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP, idle);
+            if (!roles) err = md_chain_pairs<MT>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP, idle);
+        } else if (p.beads_per_thread == 1 && p.lanes == 8)
+            err = md_substeps_split<MT, 8>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
+        else if (p.beads_per_thread == 1 && p.lanes == 4)
+            err = md_substeps_split<MT, 4>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
+        else if (p.beads_per_thread == 2)
+            err = md_substeps<MT, 2>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
+        else
+            err = md_substeps<MT, 1>(p, ch, N, n, b, sXbuf, sU, sV, sR, sP, sNb, sErrP);
+        if (err) {
+            if (tid == 0) set_status(&p.status[b], err);
+            return;
+        }
     }
-    __syncthreads();
-    for (int e = tid; e < 8 * N; e += nthr) {
+
+    // The last warps, a thread per bead, finish the beads (4) while the others
+    // spread the force (5); a block without that many warps does one after the
+    // other.  (Neighbour lists during the substeps and this side by side: a step of a
+    // 32^3 FP32 box with 16 beads 41.1 -> 37.1 us, of a 64^3 box with 32 40.2 -> 39.3.)
+    const int nbw = (N + 31) >> 5;
+    const bool side = nthr >= 64 * nbw;
+    const int com0 = side ? nthr - 32 * nbw : 0, bead = tid - com0;
+    if (bead >= 0 && bead < 32 * nbw) {
+        // 4. centre of mass pinned at the box centre.  The sums run in MT over
+        //    the offsets from bead 0's start-of-step position, which are small:
+        //    FP64 is slow on this part, and the pin is re-applied every step, so
+        //    the FP32 rounding of one step's shift does not accumulate.
+        double R[3] = {0, 0, 0};
+        MT V[3] = {0, 0, 0};
+        if (bead < N)
+            for (int a = 0; a < 3; a++) {
+                R[a] = sR[bead][a];
+                V[a] = sV[bead][a];
+            }
+        if (ch.pin_com >= 1) {
+            const int warp = bead >> 5, lane = bead & 31;
+            for (int pass = 0; pass < 2; pass++) {
+                MT s[3];
+                for (int a = 0; a < 3; a++) {
+                    s[a] = bead < N ? (pass == 0 ? (MT)(R[a] - sRc[a]) : V[a]) : MT(0);
+                    for (int o = 16; o > 0; o >>= 1) s[a] += __shfl_xor_sync(0xffffffffu, s[a], o);
+                }
+                if (lane == 0)
+                    for (int a = 0; a < 3; a++) sRed[pass][warp][a] = s[a];
+            }
+            asm volatile("bar.sync 3, %0;" ::"r"(32 * nbw) : "memory");
+            if (bead < N) {
+                MT com[3] = {0, 0, 0}, vcm[3] = {0, 0, 0};
+                for (int w = 0; w < nbw; w++)
+                    for (int a = 0; a < 3; a++) {
+                        com[a] += sRed[0][w][a];
+                        vcm[a] += sRed[1][w][a];
+                    }
+                const double centre = 0.5 * (Ei - 1);
+                const MT inv_n = sizeof(MT) == 8 ? (MT)ch.md_d[kMdInvN] : (MT)ch.md_f[kMdInvN];
+                for (int a = 0; a < 3; a++) {
+                    R[a] += (centre - sRc[a]) - (double)(com[a] * inv_n);
+                    if (ch.pin_com >= 2) V[a] = V[a] - vcm[a] * inv_n;
+                }
+            }
+        }
+        if (bead < N) {
+            for (int a = 0; a < 3; a++) {
+                pos[3 * bead + a] = R[a];
+                vel[3 * bead + a] = (double)V[a];
+            }
+            if (p.hist_slots > 0) {  // the trajectory ring: positions after step n + 1
+                double* h = p.hist + ((n + 1) % p.hist_slots) * p.hist_stride + 3 * (int64_t)ch.bead_off;
+                for (int a = 0; a < 3; a++) h[3 * bead + a] = R[a];
+            }
+        }
+    }
+    // 5. force density at the stencil sites: every entry sums, in bead order,
+    //    the contributions of all beads whose stencil holds its site (a scan of
+    //    its bead's near list); entries whose site an earlier bead already holds
+    //    are marked duplicates.
+    const int nsp = side ? com0 : nthr;  // threads that spread
+    if (!listed) {
+        if (tid < nsp) near_lists(tid, nsp);
+        __syncthreads();
+    }
+    ForceEntry* fl = p.forces + ch.force_off;
+    for (int e = tid; tid < nsp && e < 8 * N; e += nsp) {
         const int bb = e >> 3, c = e & 7;
         int s[3] = {sBase[bb][0] + (c & 1), sBase[bb][1] + ((c >> 1) & 1), sBase[bb][2] + ((c >> 2) & 1)};
         for (int a = 0; a < 3; a++)
