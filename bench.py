@@ -901,7 +901,7 @@ def run_precision(args, standalone=True):
             "roofline": {"bound": "hbm", "achieved": results["f16"]["hbm_frac"] * peak, "peak": peak, "unit": "GB/s",
                          "frac": results["f16"]["hbm_frac"], "traffic": None, "kernel": "stream-collide",
                          "peak_kind": peak_kind},
-            "e2e": None, "gpu_launches": args.steps * 2}
+            "e2e": None, "gpu_launches": args.steps}
     del faces
     torch.cuda.synchronize()
     if standalone:

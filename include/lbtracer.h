@@ -341,9 +341,10 @@ int32_t lb_set_launch(lb_ctx* ctx, int32_t kernel, int32_t threads, int32_t ctas
  *   lanes = 1 (two beads per thread), or 0 with lanes = 2: the chain-order
  *   layout -- thread t holds bead t / 2; one lane of a bead takes its bonds,
  *   the other the beads two apart, the two split the Verlet list, every pair
- *   slot masked rather than branched.  One barrier over the MD threads per
- *   substep in every layout.  lanes x ceil(largest chain / beads_per_thread)
- *   <= 512.  Used by the autotuner; drops a captured graph.  LB_ERR_ARG
+ *   slot masked rather than branched; in FP64 storage it gives chains of up
+ *   to 128 beads four warps to 32 beads instead, split by the kind of pair and
+ *   then by component.  One barrier over the MD threads per substep (two in
+ *   the FP64 split).  lanes x ceil(largest chain / beads_per_thread) <= 512.  Used by the autotuner; drops a captured graph.  LB_ERR_ARG
  *   otherwise. */
 int32_t lb_set_bead_launch(lb_ctx* ctx, int32_t lanes, int32_t beads_per_thread);
 

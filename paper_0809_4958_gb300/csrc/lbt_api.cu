@@ -410,7 +410,11 @@ int enqueue_step(lb_ctx* ctx, int64_t n)
     // so it runs alongside; with many chains the atomic tile counter balances
     // bead blocks and stream-collide blocks by itself.
     int ctas = ctx->ctas;
-    if (ctas == 0 && ctx->kernel == LB_KERNEL_STAGED) ctas = nch > 0 && nch <= ctx->sms / 8 ? ctx->sms - nch : ctx->sms;
+    if (ctx->kernel == LB_KERNEL_STAGED) {
+        if (ctas == 0) ctas = nch > 0 && nch <= ctx->sms / 8 ? ctx->sms - nch : ctx->sms;
+        // a block fills an SM; one beyond those would sit on its first tile until another block ends
+        if (ctas > ctx->sms) ctas = ctx->sms;
+    }
     CK(DISPATCH(ctx->storage, stream_collide(sp, ctx->kernel, ctx->threads, ctas, ctx->vw, ctx->stream)));
     if (timed) {
         CK(cudaEventRecordWithFlags(ctx->prof_ev[ctx->prof_used + 1], ctx->stream, evflags));

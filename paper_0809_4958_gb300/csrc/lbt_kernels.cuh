@@ -1065,7 +1065,8 @@ __device__ __forceinline__ int md_chain_pairs(const BeadParams& p, const ChainDe
 // more than their rounding: a superset, and a pair beyond the cut-off adds
 // exactly zero.  (All of a bead's work in one lane: 202 us a step of the 16-bead
 // chain in a 32^3 box and 247 of 64 beads; two lanes a bead with masked slots
-// and divisions: 298 and 371; ROLES_US.)  Flags and errors as in md_chain_pairs.
+// and divisions: 298 and 371; this: 118 and 182.)  Flags and errors as in
+// md_chain_pairs.
 constexpr int kRoleBeads = kBeadThreadsMax / 4;  // beads the four roles' warps cover
 
 template <class Idle>
