@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -211,8 +212,8 @@ struct lb_ctx {
     std::vector<size_t> zst_off;  // per zoomed box: byte offset of its coarse-sample staging (L.zstage)
     int threads = 256, ctas = 0, vw = 0;  // vw: sites per thread in stream-collide
     std::vector<int64_t> tile_prefix;  // for the current block size
-    double* host_out = nullptr;        // pinned: what a synchronising call returns (8 doubles), then the status words
-    int32_t* host_status = nullptr;
+    std::mutex host_mutex;
+    std::vector<double*> host_slots, host_free;  // pinned (host_mutex): every slot, and those no call holds (HostSlot)
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
     bool graph_parity = true;
@@ -462,19 +463,59 @@ int wait_stream(lb_ctx* ctx, int timeout_ms)
     return LB_OK;
 }
 
-// Enqueue the copy of the status words into the context's pinned memory, so
-// that the wait for the stream covers it.
-int copy_status(lb_ctx* ctx)
+// One more slot of pinned memory: 8 doubles, then the status words.
+cudaError_t add_host_slot(lb_ctx* ctx)
 {
-    CK(cudaMemcpyAsync(ctx->host_status, ctx->at<int32_t>(ctx->L.status), sizeof(int32_t) * ctx->nboxes,
+    double* slot = nullptr;
+    const cudaError_t e =
+        cudaMallocHost(reinterpret_cast<void**>(&slot), 8 * sizeof(double) + sizeof(int32_t) * ctx->nboxes);
+    if (e == cudaSuccess) {
+        ctx->host_slots.push_back(slot);
+        ctx->host_free.push_back(slot);
+    }
+    return e;
+}
+
+constexpr int kHostSlots = 4;  // made with the context; as many as there are threads in synchronising calls at once
+
+// The pinned memory of one synchronising call: several threads may wait on a
+// context, and each reads what its own copies brought.  A call that times out
+// leaves copies behind, which the next holder's copies follow in the stream.
+struct HostSlot {
+    lb_ctx* ctx;
+    double* out = nullptr;
+    explicit HostSlot(lb_ctx* c) : ctx(c)
+    {
+        std::lock_guard<std::mutex> lock(ctx->host_mutex);
+        if (ctx->host_free.empty() && add_host_slot(ctx) != cudaSuccess) return;
+        out = ctx->host_free.back();
+        ctx->host_free.pop_back();
+    }
+    ~HostSlot()
+    {
+        if (!out) return;
+        std::lock_guard<std::mutex> lock(ctx->host_mutex);
+        ctx->host_free.push_back(out);
+    }
+    HostSlot(const HostSlot&) = delete;
+    HostSlot& operator=(const HostSlot&) = delete;
+    int32_t* status() const { return reinterpret_cast<int32_t*>(out + 8); }
+};
+
+// Enqueue the copy of the status words into the call's pinned memory, so
+// that the wait for the stream covers it.
+int copy_status(lb_ctx* ctx, const HostSlot& host)
+{
+    if (!host.out) return ctx->fail(LB_ERR_CUDA, "no pinned memory for a synchronising call");
+    CK(cudaMemcpyAsync(host.status(), ctx->at<int32_t>(ctx->L.status), sizeof(int32_t) * ctx->nboxes,
                        cudaMemcpyDeviceToHost, ctx->stream));
     return LB_OK;
 }
 
 // First error among the status words copied before the wait (copy_status).
-int first_status(lb_ctx* ctx, int box)
+int first_status(lb_ctx* ctx, const HostSlot& host, int box)
 {
-    const int32_t* st = ctx->host_status;
+    const int32_t* st = host.status();
     for (int b = 0; b < ctx->nboxes; b++) {
         if ((box < 0 || box == b) && st[b] != 0) {
             char buf[96];
@@ -558,9 +599,7 @@ int32_t lb_create(const lb_box_desc* boxes, int32_t nboxes, int32_t storage, int
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
-    if (e == cudaSuccess)
-        e = cudaMallocHost(reinterpret_cast<void**>(&ctx->host_out), 8 * sizeof(double) + sizeof(int32_t) * nboxes);
-    ctx->host_status = reinterpret_cast<int32_t*>(ctx->host_out + 8);
+    for (int k = 0; k < kHostSlots && e == cudaSuccess; k++) e = add_host_slot(ctx);
     if (e != cudaSuccess) {
         g_last_error = std::string("stream/event creation: ") + cudaGetErrorString(e);
         lb_destroy(ctx);
@@ -663,7 +702,7 @@ int32_t lb_destroy(lb_ctx* ctx)
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
     if (ctx->side) cudaStreamDestroy(ctx->side);
-    if (ctx->host_out) cudaFreeHost(ctx->host_out);  // waits for copies still enqueued
+    for (double* slot : ctx->host_slots) cudaFreeHost(slot);  // waits for copies still enqueued
     delete ctx;
     return LB_OK;
 }
@@ -947,10 +986,11 @@ int32_t lb_read_fields(lb_ctx* ctx, int32_t box, int32_t what, void* dst)
         return ctx->fail(LB_ERR_ARG, "unknown field");
     }
     if (async) return LB_OK;
-    int st = copy_status(ctx);
+    const HostSlot host(ctx);
+    int st = copy_status(ctx, host);
     if (!st) st = wait_stream(ctx, kDefaultTimeoutMs);
     if (st) return st;
-    return first_status(ctx, box);
+    return first_status(ctx, host, box);
 }
 
 int32_t lb_conservation(lb_ctx* ctx, int32_t box, double* out)
@@ -962,13 +1002,15 @@ int32_t lb_conservation(lb_ctx* ctx, int32_t box, double* out)
                              ctx->nboxes, ctx->L.cons_chunks, ctx->at<double>(ctx->L.vel),
                              ctx->at<double>(ctx->L.cons_partial), ctx->at<double>(ctx->L.cons_out),
                              ctx->at<int32_t>(ctx->L.status), ctx->stream)));
-    CK(cudaMemcpyAsync(ctx->host_out, ctx->at<double>(ctx->L.cons_out) + 8 * box, 8 * sizeof(double),
-                       cudaMemcpyDeviceToHost, ctx->stream));
-    int st = copy_status(ctx);
-    if (!st) st = wait_stream(ctx, kDefaultTimeoutMs);
+    const HostSlot host(ctx);
+    int st = copy_status(ctx, host);
     if (st) return st;
-    memcpy(out, ctx->host_out, 7 * sizeof(double));
-    return first_status(ctx, box);
+    CK(cudaMemcpyAsync(host.out, ctx->at<double>(ctx->L.cons_out) + 8 * box, 8 * sizeof(double),
+                       cudaMemcpyDeviceToHost, ctx->stream));
+    st = wait_stream(ctx, kDefaultTimeoutMs);
+    if (st) return st;
+    memcpy(out, host.out, 7 * sizeof(double));
+    return first_status(ctx, host, box);
 }
 
 int32_t lb_vorticity(lb_ctx* ctx, int32_t box, int32_t lo, int32_t hi, double* out)
@@ -987,30 +1029,34 @@ int32_t lb_vorticity(lb_ctx* ctx, int32_t box, int32_t lo, int32_t hi, double* o
     const BoxDev bn = box_at_step(ctx, box);
     CK(DISPATCH(ctx->storage, fields(A, &bn, 0, bd.n3, 1, stage, ctx->stream)));
     CK(launch_vorticity(stage, ctx->storage == kF64, bd.E, lo, hi, sums, sums + 512, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->host_out, sums + 512, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    int st = copy_status(ctx);
-    if (!st) st = wait_stream(ctx, kDefaultTimeoutMs);
+    const HostSlot host(ctx);
+    int st = copy_status(ctx, host);
     if (st) return st;
-    *out = ctx->host_out[0];
-    return first_status(ctx, box);
+    CK(cudaMemcpyAsync(host.out, sums + 512, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    st = wait_stream(ctx, kDefaultTimeoutMs);
+    if (st) return st;
+    *out = host.out[0];
+    return first_status(ctx, host, box);
 }
 
 int32_t lb_sync(lb_ctx* ctx, int32_t timeout_ms)
 {
     if (!ctx) return LB_ERR_ARG;
-    int st = copy_status(ctx);
+    const HostSlot host(ctx);
+    int st = copy_status(ctx, host);
     if (!st) st = wait_stream(ctx, timeout_ms);
     if (st) return st;
-    return first_status(ctx, -1);
+    return first_status(ctx, host, -1);
 }
 
 int32_t lb_status(lb_ctx* ctx, int32_t box, int32_t* status)
 {
     if (!ctx || !status || box < 0 || box >= ctx->nboxes) return LB_ERR_ARG;
-    int st = copy_status(ctx);
+    const HostSlot host(ctx);
+    int st = copy_status(ctx, host);
     if (!st) st = wait_stream(ctx, kDefaultTimeoutMs);
     if (st) return st;
-    *status = ctx->host_status[box];
+    *status = host.status()[box];
     return LB_OK;
 }
 
