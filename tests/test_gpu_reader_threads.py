@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 def test_conservation_of_different_boxes_from_several_threads():
     from paper_0809_4958_gb300 import lbtracer as lbt
     lbt.load()
-    sizes = [8, 12, 16, 20, 24, 28]
+    sizes = [8, 16, 24, 32, 40, 48]
     tr = lbt.Tracers([lbt.box_desc(E, 0.8, periodic=(True, True, True)) for E in sizes], 0)
     for b, E in enumerate(sizes):
         tr.lb_init(b, np.full((3, E, E, E), 0.01 * (b + 1)))
