@@ -1555,12 +1555,16 @@ int32_t lb_mlp_forward(const void* params, int32_t K, const void* X, int64_t row
                        "lb_mlp_forward");
 }
 
-// The gradient and the loss go straight to device memory; anything else takes a copy behind the kernels.
+// The gradient and the loss go straight to device memory that is aligned for
+// them; anything else takes a copy behind the kernels.
 static cudaError_t train_rows(void* ws, int32_t K, int64_t batch_rows, const void* X, const float* T, int64_t rows,
                               float* grad_out, double* loss_out, bool adam, float lr, int64_t t, cudaStream_t s)
 {
     const MlpTrain W = mlp_train_layout(K, batch_rows);
-    const bool gd = grad_out && is_device_ptr(grad_out), ld = loss_out && is_device_ptr(loss_out);
+    auto direct = [](const void* q, size_t size) {
+        return q && reinterpret_cast<uintptr_t>(q) % size == 0 && is_device_ptr(q);
+    };
+    const bool gd = direct(grad_out, sizeof(float)), ld = direct(loss_out, sizeof(double));
     const float* f = reinterpret_cast<const float*>(ws);
     cudaError_t e = mlp_train(reinterpret_cast<unsigned char*>(ws), W, X, T, rows, gd ? grad_out : nullptr,
                               ld ? loss_out : nullptr, adam, lr, t, s);

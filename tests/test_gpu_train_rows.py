@@ -58,3 +58,28 @@ def test_gradient_at_tile_edges(K, rows, offset):
     g2 = got[32 * 128 + 128:32 * 128 + 128 + 128 * 128].view(128, 128)
     new = (m2 - 1e-3 * g2 / (g2.abs() + 1e-8)).T
     assert float((w2.float() - new).abs().max()) <= 2.0 ** -8 * float(new.abs().max()) + 1e-5
+
+
+def test_loss_on_a_four_byte_boundary():
+    """The loss (8 bytes) may go anywhere in device memory, between floats too."""
+    import torch
+
+    from paper_0809_4958_gb300 import inputs, lbtracer as lbt
+    lib = lbt.load()
+    K, rows = 8, 300
+    up = lbt.Upsampler(K=K, batch_rows=rows, master=inputs.mlp_init(3, K))
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.randn((rows, 32), device="cuda", generator=g).to(torch.bfloat16)
+    X[:, 24:] = 0
+    T = torch.randn((rows, 3 * K), device="cuda", generator=g)
+    _, loss = up.grad(X, T)
+    want = float(loss)
+    buf = torch.zeros(4, dtype=torch.float32, device="cuda")
+    out = torch.zeros(up.nmaster(), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    rc = lib.lb_mlp_grad(up.ws.data_ptr(), K, rows, X.data_ptr(), T.data_ptr(), rows, out.data_ptr(),
+                         buf.data_ptr() + 4, up.stream.cuda_stream)
+    assert rc == 0
+    torch.cuda.synchronize()
+    assert float(np.frombuffer(buf.cpu().numpy()[1:3].tobytes())[0]) == want
+    assert float(buf[0]) == 0.0 and float(buf[3]) == 0.0
