@@ -1635,38 +1635,61 @@ __global__ void __launch_bounds__(kForcedThreads) k_forced(ForcedParams p)
             if (fe.site >= 0) {
                 site = fe.site;
                 const int x = site % Ei, y = (site / Ei) % Ei, z = site / (Ei * Ei);
-                A dr, j[3];
+                A dr, j[3], F[3], u[3];
                 pull_site<ST, true>(Ab, n3, Ei, per, x, y, z, val);
-                site_moments<A, 1>([&](int i) { return val[i]; }, dr, j);
-                const A rho = A(1) + dr, inv = fast_inverse(rho);
-                A F[3], u[3];
-                for (int a = 0; a < 3; a++) {
-                    F[a] = rho * (A)p.chain_accel[4 * chain + a] + (A)fe.g[a];
-                    u[a] = ratio(j[a] + A(0.5) * F[a], rho, inv);
-                }
-                const A om = A(1) / (A)bd.tau, om1 = A(1) - om, sf = A(1) - A(0.5) * om;
-                const A usq = A(1.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-                const A uF3 = A(3) * (u[0] * F[0] + u[1] * F[1] + u[2] * F[2]);
-                // by opposite pairs: om (drho + rho (4.5 cu^2 - 1.5 u^2)) + sf (9 cu cF - 3 u.F) in common,
-                // om rho 3 cu + sf 3 cF changing sign
-                const A even0 = om * (dr - rho * usq) - sf * uF3, omr = om * rho;
-                val[0] = om1 * val[0] + wgt<A>(0) * even0;
+                if constexpr (sizeof(A) == 8) {
+                    // the FP64 pipe runs two lanes a clock: moments and populations by opposite pairs, one reciprocal
+                    site_moments<A, 1>([&](int i) { return val[i]; }, dr, j);
+                    const A rho = A(1) + dr, inv = fast_inverse(rho);
+                    for (int a = 0; a < 3; a++) {
+                        F[a] = rho * (A)p.chain_accel[4 * chain + a] + (A)fe.g[a];
+                        u[a] = ratio(j[a] + A(0.5) * F[a], rho, inv);
+                    }
+                    const A om = A(1) / (A)bd.tau, om1 = A(1) - om, sf = A(1) - A(0.5) * om;
+                    const A usq = A(1.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+                    const A uF3 = A(3) * (u[0] * F[0] + u[1] * F[1] + u[2] * F[2]);
+                    // by opposite pairs: om (drho + rho (4.5 cu^2 - 1.5 u^2)) + sf (9 cu cF - 3 u.F) in common,
+                    // om rho 3 cu + sf 3 cF changing sign
+                    const A even0 = om * (dr - rho * usq) - sf * uF3, omr = om * rho;
+                    val[0] = om1 * val[0] + wgt<A>(0) * even0;
 #pragma unroll
-                for (int i = 1; i < kQ; i += 2) {
-                    A cu = A(0), cF = A(0);
-                    bool some = false;
+                    for (int i = 1; i < kQ; i += 2) {
+                        A cu = A(0), cF = A(0);
+                        bool some = false;
 #pragma unroll
-                    for (int a = 0; a < 3; a++)
-                        if (cvec(i, a)) {
-                            const A su = cvec(i, a) > 0 ? u[a] : -u[a], sF = cvec(i, a) > 0 ? F[a] : -F[a];
-                            cu = some ? cu + su : su;
-                            cF = some ? cF + sF : sF;
-                            some = true;
-                        }
-                    const A w = wgt<A>(i);
-                    const A even = even0 + cu * (A(4.5) * omr * cu + A(9) * sf * cF), odd = A(3) * (omr * cu + sf * cF);
-                    val[i] = om1 * val[i] + w * (even + odd);
-                    val[i + 1] = om1 * val[i + 1] + w * (even - odd);
+                        for (int a = 0; a < 3; a++)
+                            if (cvec(i, a)) {
+                                const A su = cvec(i, a) > 0 ? u[a] : -u[a], sF = cvec(i, a) > 0 ? F[a] : -F[a];
+                                cu = some ? cu + su : su;
+                                cF = some ? cF + sF : sF;
+                                some = true;
+                            }
+                        const A w = wgt<A>(i);
+                        const A even = even0 + cu * (A(4.5) * omr * cu + A(9) * sf * cF), odd = A(3) * (omr * cu + sf * cF);
+                        val[i] = om1 * val[i] + w * (even + odd);
+                        val[i + 1] = om1 * val[i + 1] + w * (even - odd);
+                    }
+                } else {
+                    // FP32: population by population.  The chain amplifies a last bit of these sites from step to
+                    // step, so their rounding is kept; the time hides behind the stream-collide.
+                    moments<A>(val, dr, j);
+                    const A rho = A(1) + dr;
+                    for (int a = 0; a < 3; a++) {
+                        F[a] = rho * (A)p.chain_accel[4 * chain + a] + (A)fe.g[a];
+                        u[a] = (j[a] + A(0.5) * F[a]) / rho;
+                    }
+                    const A om = A(1) / (A)bd.tau;
+                    const A usq = A(1.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+                    const A uF = u[0] * F[0] + u[1] * F[1] + u[2] * F[2];
+#pragma unroll
+                    for (int i = 0; i < kQ; i++) {
+                        const A w = wgt<A>(i);
+                        const A cu = cvec(i, 0) * u[0] + cvec(i, 1) * u[1] + cvec(i, 2) * u[2];
+                        const A cF = cvec(i, 0) * F[0] + cvec(i, 1) * F[1] + cvec(i, 2) * F[2];
+                        const A deq = w * (dr + rho * (A(3) * cu + A(4.5) * cu * cu - usq));
+                        val[i] += om * (deq - val[i]);
+                        val[i] += (A(1) - A(0.5) * om) * w * (A(3) * (cF - uF) + A(9) * cu * cF);
+                    }
                 }
             }
         }
