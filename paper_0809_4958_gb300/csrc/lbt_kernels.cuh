@@ -1802,7 +1802,10 @@ __global__ void __launch_bounds__(kFieldsThreads) k_fields(const typename Stor<S
     const bool px = per & 1, py = per & 2, pz = per & 4;
     const int n3 = (int)bd.n3, lane = threadIdx.x & 31;
     // A read-out of many boxes is many small launches: each is a programmatic
-    // dependent of the one before and lets the next be scheduled at once
+    // dependent of the one before and lets the next be scheduled at once.  The
+    // first may follow the step whose stores it reads and be resident while they
+    // are made, so the populations are not read-only for this grid's lifetime:
+    // ordinary loads, which the wait orders, not the non-coherent path.
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int G = blockIdx.x * kFieldsThreads + threadIdx.x; G < n3 / VW; G += gridDim.x * kFieldsThreads) {
@@ -1823,14 +1826,14 @@ __global__ void __launch_bounds__(kFieldsThreads) k_fields(const typename Stor<S
         for (int i = 0; i < kQ; i++, pop += n3) {
             const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
             const E* src = pop + ((cy > 0 ? ym : (cy < 0 ? yp : 0)) + (cz > 0 ? zm : (cz < 0 ? zp : 0)));
-            v[i].raw = ld_nc(reinterpret_cast<const Raw*>(src));
+            v[i].raw = *reinterpret_cast<const Raw*>(src);
             // an x-face site takes its own element in the neighbour's place ...
-            if (cx > 0 && load_l) nb[i] = __ldg(edge_l ? pop : src + nl);
-            if (cx < 0 && load_r) nb[i] = __ldg(edge_r ? pop + VW - 1 : src + nr);
+            if (cx > 0 && load_l) nb[i] = *(edge_l ? pop : src + nl);
+            if (cx < 0 && load_r) nb[i] = *(edge_r ? pop + VW - 1 : src + nr);
             // ... or in the place inside the group its shifted value comes from
-            if (cx > 0 || (cx == 0 && i > 0)) own[i] = edge_r ? __ldg(pop + VW - 1) : E(0);
-            if (cx < 0) own[i] = edge_l ? __ldg(pop) : E(0);
-            if (cx == 0 && i > 0 && edge_l) own[i] = __ldg(pop);
+            if (cx > 0 || (cx == 0 && i > 0)) own[i] = edge_r ? pop[VW - 1] : E(0);
+            if (cx < 0) own[i] = edge_l ? *pop : E(0);
+            if (cx == 0 && i > 0 && edge_l) own[i] = *pop;
         }
         if constexpr (kShuffle) {  // n3 / VW is a multiple of 32: whole warps take part
 #pragma unroll
