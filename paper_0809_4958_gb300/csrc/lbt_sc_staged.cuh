@@ -828,7 +828,7 @@ __device__ __forceinline__ void staged_tile_fluct_pair(const SCParams& p, const 
                 }
             }
         }
-        f[i] = v;  // boundary lanes: finite, multiplied by zero below
+        f[i] = v;  // boundary lanes: not used
     }
     __syncwarp();
     if ((tid & 31) == 0) mbar_arrive(empty);  // this warp is done with the stage
@@ -913,8 +913,8 @@ __device__ __forceinline__ void staged_tile_fluct_pair(const SCParams& p, const 
         m[8] = fma2(f2(-2.f), f[6], add2(sz, tz));
         m[11] = sub2(sz, tz);
     }
-    // relaxed moments plus noise, over their norms; none on boundary sites
-    const float2 keep = make_float2(bnd0 ? 0.f : 1.f, bnd1 ? 0.f : 1.f);
+    // relaxed moments plus noise, over their norms; none on boundary sites (selected, not multiplied by zero: what a
+    // boundary site pulled means nothing, its density may have no square root and its values may be infinite)
     const FluctDev& fd = p.fluct[th.box];
     const uint32_t k0 = (uint32_t)fd.seed, k1 = (uint32_t)(fd.seed >> 32);
 #pragma unroll
@@ -930,7 +930,8 @@ __device__ __forceinline__ void staged_tile_fluct_pair(const SCParams& p, const 
             if (4 * blk + w < 15) {
                 const float2 xi = make_float2(unit_uniform_t<float>(xa[w]), unit_uniform_t<float>(xb[w]));
                 float2& mk = m[4 * blk + w];
-                mk = mul2(keep, fma2(f2(gk[w]), mk, mul2(mul2(f2(ak[w]), srho), xi)));
+                const float2 relaxed = fma2(f2(gk[w]), mk, mul2(mul2(f2(ak[w]), srho), xi));
+                mk = make_float2(bnd0 ? 0.f : relaxed.x, bnd1 ? 0.f : relaxed.y);
             }
     }
     // back to the populations: equilibrium + w (even part +- odd part)
