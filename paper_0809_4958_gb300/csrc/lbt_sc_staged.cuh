@@ -757,8 +757,11 @@ __device__ __forceinline__ void staged_tile_fluct(const SCParams& p, const Stage
         }
         int pp, qq;
         const int fc = owning_face(x, y, z, Ei, per, pp, qq);
+        float res[3];
+        load_mlp_residual(p, bd, th.mlp_s, fc, pp, qq, res);
         R ub[3];
         boundary_velocity<R>(reinterpret_cast<const R*>(p.ring), p.ring_slot_elems, bd, fc, pp, qq, tw, ub);
+        add_mlp_residual<R>(p, bd, res, ub);
         const A dr = th.drho_b, rb = A(1) + dr;
         const A u0 = (A)ub[0], u1 = (A)ub[1], u2 = (A)ub[2];
         const A usq = A(1.5) * (u0 * u0 + u1 * u1 + u2 * u2);
