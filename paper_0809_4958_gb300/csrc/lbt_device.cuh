@@ -161,10 +161,12 @@ __device__ __forceinline__ float unit_uniform_t<float>(uint32_t v)
 }
 
 // 1 / x by the hardware's approximation: in FP32 PTX rcp.approx.ftz.f32 (at
-// most one ulp), in FP64 about 20 bits refined by one third-order step
-// x' = x (1 + e + e^2), e = 1 - a x, which leaves e^3; without the branch of the
-// library's division, so that independent reciprocals interleave (an FP64
-// instruction takes some 64 cycles to its result).
+// most one ulp), in FP64 about 20 bits refined by one step of Householder's
+// third-order iteration y' = y (1 + e + e^2), e = 1 - x y, which leaves e^3
+// (within one ulp); without the branch of the library's division, so that
+// independent reciprocals interleave (an FP64 instruction takes some 64 cycles
+// to its result).  For x and 1 / x in the normal range; zero, infinite and
+// subnormal x give NaN in FP64, and a subnormal 1 / x is flushed to zero.
 __device__ __forceinline__ double fast_inverse(double x)
 {
     double y;

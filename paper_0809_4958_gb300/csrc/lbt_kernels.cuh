@@ -242,16 +242,18 @@ __global__ void __launch_bounds__(256) k_stream_collide(SCParams p)
 // Per-site helpers for the scalar kernels (bead gather, forced re-collision,
 // fields).
 // ---------------------------------------------------------------------------
-// j / rho from r = 1 / rho, the product corrected by its own residual (within
-// one ulp), so that the three components share one reciprocal; the division
-// itself where the result is not finite.
+// j / rho from r = 1 / rho, the product corrected by its own residual
+// (Markstein's quotient; within one ulp, two where |j| is near the smallest
+// normal number), so that the three components share one reciprocal; the
+// division itself where the result is not finite, and where the reciprocal has
+// been flushed to zero (rho beyond a quarter of the largest number).
 static __device__ __noinline__ double slow_ratio(double j, double rho) { return j / rho; }
 static __device__ __noinline__ float slow_ratio(float j, float rho) { return j / rho; }
 template <class A>
 __device__ __forceinline__ A ratio(A j, A rho, A r)
 {
     const A q = j * r, t = fma(fma(-q, rho, j), r, q);
-    return isfinite(t) ? t : slow_ratio(j, rho);
+    return isfinite(t) && r != A(0) ? t : slow_ratio(j, rho);
 }
 // Density deviation and (WHAT = 1) momentum of one site from its populations,
 // by opposite pairs: their sums make the density, their differences the
