@@ -1807,7 +1807,7 @@ __global__ void __launch_bounds__(kFieldsThreads) k_fields(const typename Stor<S
     // dependent of the one before and lets the next be scheduled at once.  The
     // first may follow the step whose stores it reads and be resident while they
     // are made, so the populations are not read-only for this grid's lifetime:
-    // ordinary loads, which the wait orders, not the non-coherent path.
+    // ordinary loads, which the wait orders (ld_ordered), not the read-only path.
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int G = blockIdx.x * kFieldsThreads + threadIdx.x; G < n3 / VW; G += gridDim.x * kFieldsThreads) {
@@ -1828,14 +1828,14 @@ __global__ void __launch_bounds__(kFieldsThreads) k_fields(const typename Stor<S
         for (int i = 0; i < kQ; i++, pop += n3) {
             const int cx = cvec(i, 0), cy = cvec(i, 1), cz = cvec(i, 2);
             const E* src = pop + ((cy > 0 ? ym : (cy < 0 ? yp : 0)) + (cz > 0 ? zm : (cz < 0 ? zp : 0)));
-            v[i].raw = *reinterpret_cast<const Raw*>(src);
+            v[i].raw = ld_ordered(reinterpret_cast<const Raw*>(src));
             // an x-face site takes its own element in the neighbour's place ...
-            if (cx > 0 && load_l) nb[i] = *(edge_l ? pop : src + nl);
-            if (cx < 0 && load_r) nb[i] = *(edge_r ? pop + VW - 1 : src + nr);
+            if (cx > 0 && load_l) nb[i] = ld_ordered(edge_l ? pop : src + nl);
+            if (cx < 0 && load_r) nb[i] = ld_ordered(edge_r ? pop + VW - 1 : src + nr);
             // ... or in the place inside the group its shifted value comes from
-            if (cx > 0 || (cx == 0 && i > 0)) own[i] = edge_r ? pop[VW - 1] : E(0);
-            if (cx < 0) own[i] = edge_l ? *pop : E(0);
-            if (cx == 0 && i > 0 && edge_l) own[i] = *pop;
+            if (cx > 0 || (cx == 0 && i > 0)) own[i] = edge_r ? ld_ordered(pop + VW - 1) : E(0);
+            if (cx < 0) own[i] = edge_l ? ld_ordered(pop) : E(0);
+            if (cx == 0 && i > 0 && edge_l) own[i] = ld_ordered(pop);
         }
         if constexpr (kShuffle) {  // n3 / VW is a multiple of 32: whole warps take part
 #pragma unroll
