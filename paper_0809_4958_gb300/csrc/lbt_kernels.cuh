@@ -1063,13 +1063,35 @@ __device__ __forceinline__ int md_chain_pairs(const BeadParams& p, const ChainDe
 // skipped where no lane is within the cut-off).  The forces meet in shared
 // memory; then roles 0 - 2 advance component x, y and z of every bead.  Two
 // barriers a substep.  Groups of 32 beads rotate the roles over the quarters.
-// Lists come from FP32 copies of the positions with a radius larger by 1e-5,
-// more than their rounding: a superset, and a pair beyond the cut-off adds
-// exactly zero.  (All of a bead's work in one lane: 202 us a step of the 16-bead
+// Lists come from FP32 copies of the positions (list_copy) with a radius larger
+// by more than their rounding (list_reach2): a superset, and a pair beyond the
+// cut-off adds exactly zero.  (All of a bead's work in one lane: 202 us a step of the 16-bead
 // chain in a 32^3 box and 247 of 64 beads; two lanes a bead with masked slots
 // and divisions: 298 and 371; this: 118 and 182.)  Flags and errors as in
 // md_chain_pairs.
 constexpr int kRoleBeads = kBeadThreadsMax / 4;  // beads the four roles' warps cover
+
+// FP32 copy of a position (relative to bead 0) with the largest magnitude of its coordinates.
+__device__ __forceinline__ float4 list_copy(double x, double y, double z)
+{
+    const float a = (float)x, b = (float)y, c = (float)z;
+    return make_float4(a, b, c, fmaxf(fabsf(a), fmaxf(fabsf(b), fabsf(c))));
+}
+// Square of the FP32 distance that every pair within rl is below: a coordinate
+// is off by 2^-24 of its magnitude, those of a partner within rl are at most
+// top + rl, so the difference vector is off by sqrt(3) 2^-23 (top + rl) =
+// 2.1e-7 (top + rl); the roundings of the differences, squares and of rl itself
+// add less than 1e-6 rl.
+__device__ __forceinline__ float list_reach2(float rl, float top)
+{
+    const float r = fmaf(3e-7f, top, rl * (1.0f + 4e-6f));
+    return r * r;
+}
+__device__ __forceinline__ bool list_near(const float4& x, const float4& q, float reach2)
+{
+    const float dx = x.x - q.x, dy = x.y - q.y, dz = x.z - q.z;
+    return dx * dx + dy * dy + dz * dz < reach2;
+}
 
 template <class Idle>
 __device__ __forceinline__ int md_chain_roles(const BeadParams& p, const ChainDev& ch, int N, int64_t n, int b,
@@ -1091,11 +1113,11 @@ __device__ __forceinline__ int md_chain_roles(const BeadParams& p, const ChainDe
     const double R02 = mc[kMdR02], invR02 = mc[kMdInvR02], kf = mc[kMdKf], sig2 = mc[kMdSig2], rc2 = mc[kMdRc2],
                  e24 = mc[kMdE24];
     const bool wca = ch.eps > 0.0;
-    const float rl2 = (float)mc[kMdRl2] * (1.0f + 2e-5f);
+    const float rl = sqrtf((float)mc[kMdRl2]);
     const double skin_c2 = mc[kMdSkinComp2];
     if (tid < 2) sErrP[tid] = 0;
     if (tid == 0) sErrB = 0;
-    for (int g = tid; g < N; g += nthr) sXf[g] = make_float4((float)sX4[g].x, (float)sX4[g].y, (float)sX4[g].z, 0.f);
+    for (int g = tid; g < N; g += nthr) sXf[g] = list_copy(sX4[g].x, sX4[g].y, sX4[g].z);
     for (int e = tid; e < 4 * 3 * (kRoleBeads + 2); e += nthr) (&sF[0][0][0])[e] = 0.0;
     __syncthreads();
     // lists from the start positions: eight threads per bead scan every eighth partner and merge
@@ -1108,12 +1130,11 @@ __device__ __forceinline__ int md_chain_roles(const BeadParams& p, const ChainDe
             uint32_t m = 0;  // bit k: partner r + 8 k (N <= 256)
             if (act) {
                 const float4 xb = sXf[bb];
+                const float reach2 = list_reach2(rl, xb.w);
                 for (int k = 0, p2 = r; p2 < N; k++, p2 += 8) {
                     const int dd = p2 - bb;
                     if (dd >= -2 && dd <= 2) continue;
-                    const float4 q = sXf[p2];
-                    const float dx = xb.x - q.x, dy = xb.y - q.y, dz = xb.z - q.z;
-                    if (dx * dx + dy * dy + dz * dz < rl2) m |= 1u << k;
+                    if (list_near(xb, sXf[p2], reach2)) m |= 1u << k;
                 }
             }
             const int cnt = __popc(m);
@@ -1236,17 +1257,16 @@ __device__ __forceinline__ int md_chain_roles(const BeadParams& p, const ChainDe
                 // publish Xn; any flag: stop on an error, or rebuild the lists
                 if (bar_or(1, nmd, stretched || moved)) {
                     if (sErrP[sub & 1]) break;
-                    if (own && role == 3) sXf[g] = make_float4((float)Xn[4 * g], (float)Xn[4 * g + 1], (float)Xn[4 * g + 2], 0.f);
+                    if (own && role == 3) sXf[g] = list_copy(Xn[4 * g], Xn[4 * g + 1], Xn[4 * g + 2]);
                     sync_md(2);
                     if (own && role == 2 && wca) {
                         const float4 xb = sXf[g];
+                        const float reach2 = list_reach2(rl, xb.w);
                         int cnt = 0;
                         for (int p2 = 0; p2 < N; p2++) {
                             const int dd = p2 - g;
                             if (dd >= -2 && dd <= 2) continue;
-                            const float4 q = sXf[p2];
-                            const float ex = xb.x - q.x, ey = xb.y - q.y, ez = xb.z - q.z;
-                            if (ex * ex + ey * ey + ez * ez < rl2) {
+                            if (list_near(xb, sXf[p2], reach2)) {
                                 if (cnt < kMaxTasks) sNb[g][cnt] = (unsigned char)p2;
                                 cnt++;
                             }

@@ -27,9 +27,25 @@ __global__ void k_widen(const float* x, double* y, int n)
     if (i < n) y[i] = lbt::widen(x[i]);
 }
 
+// pairs a, b (n x 3): listed within the radius rl of a?
+__global__ void k_listed(const double* a, const double* b, const double* rl2, float* y, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float4 x = lbt::list_copy(a[3 * i], a[3 * i + 1], a[3 * i + 2]);
+    const float4 q = lbt::list_copy(b[3 * i], b[3 * i + 1], b[3 * i + 2]);
+    y[i] = lbt::list_near(x, q, lbt::list_reach2(sqrtf((float)rl2[i]), x.w)) ? 1.f : 0.f;
+}
+
 }  // namespace
 
 extern "C" {
+
+int t_listed(const double* a, const double* b, const double* rl2, float* y, int n)
+{
+    k_listed<<<(n + 255) / 256, 256>>>(a, b, rl2, y, n);
+    return cudaDeviceSynchronize();
+}
 
 int t_inverse_f64(const double* x, double* y, int n)
 {

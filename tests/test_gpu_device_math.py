@@ -29,9 +29,10 @@ def dev(tmp_path_factory):
 
     def call(name, out_dtype, *arrays):
         ts = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in arrays]
-        y = torch.zeros(len(arrays[0]), dtype=torch.float64 if out_dtype == np.float64 else torch.float32, device="cuda")
+        n = len(arrays[-1])
+        y = torch.zeros(n, dtype=torch.float64 if out_dtype == np.float64 else torch.float32, device="cuda")
         torch.cuda.synchronize()
-        args = [ctypes.c_void_p(t.data_ptr()) for t in ts] + [ctypes.c_void_p(y.data_ptr()), len(arrays[0])]
+        args = [ctypes.c_void_p(t.data_ptr()) for t in ts] + [ctypes.c_void_p(y.data_ptr()), n]
         assert getattr(lib, name)(*args) == 0
         return y.cpu().numpy()
 
@@ -118,3 +119,28 @@ def test_widening_is_exact(dev):
     nan = np.isnan(want)
     assert np.isnan(got[nan]).all()
     assert np.array_equal(got[~nan].view(np.uint64), want[~nan].view(np.uint64))
+
+
+@pytest.mark.parametrize("rl", [0.36, 1.4224, 4.0])
+@pytest.mark.parametrize("span", [1.0, 60.0, 200.0, 5000.0])
+def test_neighbour_lists_hold_every_pair_within_their_radius(dev, rl, span):
+    """The FP32 lists of FP64 chains: a pair just inside the FP64 radius is
+    listed however far from bead 0 it lies (a margin of 1e-5 of the radius
+    alone misses pairs from some 128 units on), one clearly outside is not."""
+    rng = np.random.default_rng(5)
+    n = 1 << 18
+    a = rng.uniform(-span, span, (n, 3))
+    e = rng.standard_normal((n, 3))
+    e /= np.linalg.norm(e, axis=1)[:, None]
+    inside = a + rl * (1 - 1e-9) * e
+    far = a + (rl * (1 + 2e-5) + 2e-6 * span) * e
+    r2 = np.full(n, rl * rl)
+    keep = ((inside - a) ** 2).sum(1) < r2
+    assert keep.mean() > 0.9
+    got = dev("t_listed", np.float32, a, inside, r2)
+    f = lambda x: x.astype(np.float32)  # noqa: E731
+    d = f(a) - f(inside)
+    former = (d * d).sum(1) < np.float32(rl * rl) * np.float32(1 + 2e-5)
+    print("span %g, radius %g: %d of %d pairs missed by a relative margin alone" % (span, rl, (~former[keep]).sum(), keep.sum()))
+    assert (got[keep] == 1).all()
+    assert (dev("t_listed", np.float32, a, far, r2) == 0).all()
