@@ -155,7 +155,10 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     float colsum[OH];  // this thread's share of sum_r dY[r][o], FP32
 #pragma unroll
     for (int c = 0; c < OH; c++) colsum[c] = 0.f;
-    float ls = 0.f, le = 0.f;  // sum of squares as an unevaluated sum of two words
+    // sum of the squares of Y - T: FP32 triple words, no less exact than an FP64 sum (Sum3); what their range does not
+    // hold goes to an FP64 one
+    Sum3 sq;
+    double sq_far = 0.0;
     uint32_t phase = 0;
     bool ok = true, first = true;
     const bool t_vec = (reinterpret_cast<uintptr_t>(T) & 15) == 0;
@@ -244,7 +247,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             tc_commit(&sm.bar);
         }
         if (!wait_mma()) break;
-        // dY = 2 (Y - T) scale, the loss and the column sums in FP32, dY in bf16 for the MMAs
+        // Y - T; dY = 2 (Y - T) scale, its column sums in FP32, itself in bf16 for the MMAs
         {
             uint32_t v[OH];
             tc_ld16_nowait(trow + kColWork + half * OH, v);
@@ -253,17 +256,12 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             uint32_t pk[OH / 2];
 #pragma unroll
             for (int c = 0; c < OH; c++) {
-                const float d = in && half * OH + c < NOUT ? __uint_as_float(v[c]) - t[c] : 0.f;
-                const float sq = d * d, lo = fmaf(d, d, -sq);
-                const float s = ls + sq, bb = s - ls;
-                le += ((ls - (s - bb)) + (sq - bb)) + lo;
-                ls = s;
-                t[c] = 2.f * d * scale;
-                colsum[c] += t[c];
+                t[c] = in && half * OH + c < NOUT ? __uint_as_float(v[c]) - t[c] : 0.f;
+                colsum[c] += 2.f * t[c] * scale;
             }
 #pragma unroll
             for (int c = 0; c < OH / 2; c++) {
-                const __nv_bfloat162 p = __floats2bfloat162_rn(t[2 * c], t[2 * c + 1]);
+                const __nv_bfloat162 p = __floats2bfloat162_rn(2.f * t[2 * c] * scale, 2.f * t[2 * c + 1] * scale);
                 pk[c] = *reinterpret_cast<const uint32_t*>(&p);
             }
 #pragma unroll
@@ -280,6 +278,20 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             // dW3 += H2^T dY, while the epilogue of dH2 runs
             mma_chain<kTcRows / 16>(tmem + kColW3, a2, 2 * kR128, kR128, kCore, ay, 2 * kRNP, kRNP, kCore,
                                     tc_idesc(kMlpHidden, NP, true, true), !first);
+        }
+        // the loss, meanwhile: squares of 24-bit values are exact in two words from 2^-51 on, and far from overflow below 2^50
+#pragma unroll
+        for (int c = 0; c < OH; c += 2) {
+            float d[2];
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                d[k] = t[c + k];
+                if (!(fabsf(d[k]) >= 0x1p-51f && fabsf(d[k]) < 0x1p50f)) {
+                    if (d[k] != 0.f) sq_far += (double)d[k] * (double)d[k];
+                    d[k] = 0.f;
+                }
+            }
+            sq.add_square(make_float2(d[0], d[1]));
         }
         if (!wait_mma()) break;
         masked_epilogue(trow + kColWork + half * kTrHalf, sm.h2, sm.dz2, m, half * kTrHalf);
@@ -346,7 +358,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         for (int o = 16; o > 0; o >>= 1) colsum[c] += __shfl_xor_sync(0xffffffffu, colsum[c], o);
         if (lane == 0) sm.col[q][half * OH + c] = colsum[c];
     }
-    double loss = (double)ls + (double)le;
+    double loss = sq.value() + sq_far;
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
     if (lane == 0) sm.loss[warp] = loss;
     tc_fence_before();
