@@ -253,6 +253,7 @@ MlpTrain mlp_train_layout(int K, int64_t B)
     const int64_t tiles = (B + 127) / 128, parts = tiles < kMlpMaxPartials ? tiles : kMlpMaxPartials;
     W.partial = take(parts * P);   // gradient of each block of the training kernel
     W.loss_part = take(2 * parts);
+    W.late = take(parts);  // int flags of the blocks
     W.loss = take(2);  // one double
     W.params_byte = o * 4;
     W.bytes = al256(W.params_byte + W.L.bytes);

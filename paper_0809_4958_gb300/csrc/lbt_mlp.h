@@ -28,7 +28,7 @@ struct MlpTrain {
     MlpLayout L;
     int K;
     int64_t batch;
-    size_t master, m, v, grad, partial, loss_part, loss;
+    size_t master, m, v, grad, partial, loss_part, late, loss;
     size_t params_byte, bytes;
 };
 

@@ -100,13 +100,14 @@ __device__ __forceinline__ void mma_chain(uint32_t d, uint32_t a, uint32_t a_ste
 }
 
 // partial: [gridDim.x][nmaster] gradient partials in master layout, loss_part
-// [gridDim.x].  scale = 1 / (rows NOUT).
+// and late [gridDim.x]: late is 1 where an MMA did not complete in time, and
+// the partial is not to be used.  scale = 1 / (rows NOUT).
 template <int NOUT>
 __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloat16* __restrict__ X,
                                                                 const float* __restrict__ T, int64_t rows,
                                                                 const unsigned char* __restrict__ params, MlpLayout L,
                                                                 float scale, float* __restrict__ partial,
-                                                                double* __restrict__ loss_part)
+                                                                double* __restrict__ loss_part, int* __restrict__ late)
 {
     using Sm = TrSmem<NOUT>;
     constexpr int NP = Sm::kNP, OH = NP / 2;  // output columns of a thread
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         first = false;
         if (!wait_mma()) break;  // every operand read: the next tile may be staged
     }
-    if (!ok) tc_wait(&sm.bar, phase ^ 1u);  // let an MMA still in flight finish (bounded); the loss below says what happened
+    if (!ok) tc_wait(&sm.bar, phase ^ 1u);  // let an MMA still in flight finish (bounded); `late` below says what happened
 
     // the block's partial in master layout; lane m is the row of each D
     float* P = partial + (int64_t)blockIdx.x * L.nmaster;
@@ -368,7 +369,8 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     if (tid == 0) {
         double t = 0.0;
         for (int w = 0; w < kTrThreads / 32; w++) t += sm.loss[w];
-        loss_part[blockIdx.x] = ok ? t * scale : __longlong_as_double(0x7ff8000000000000ll);  // NaN: an MMA timed out
+        loss_part[blockIdx.x] = t * scale;
+        late[blockIdx.x] = !ok;
     }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTrCols) : "memory");
@@ -377,7 +379,10 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
 // Gradient = the blocks' partials added in a fixed order; then (ADAM) Adam on
 // the master weights and the bf16 / FP32 inference copy of what changed.  A
 // block takes 32 parameters (a lane each) in eight slices of the partials.
+// Where a block's MMAs were late, gradient and loss are NaN and the weights and
+// their moments stay as they are.
 constexpr int kRdSlices = 8;
+static_assert(kMlpMaxPartials <= 32 * kRdSlices, "a thread per block's flag");
 
 struct AdamArgs {
     float *master, *m, *v;
@@ -402,8 +407,8 @@ __device__ __forceinline__ void export_one(int64_t e, float w, const MlpLayout& 
 
 template <bool ADAM>
 __global__ void __launch_bounds__(32 * kRdSlices) k_mlp_reduce(const float* __restrict__ partial,
-                                                               const double* __restrict__ loss_part, int nparts,
-                                                               MlpLayout L, float* __restrict__ grad, float* grad_out,
+                                                               const double* __restrict__ loss_part,
+                                                               const int* __restrict__ late, int nparts, MlpLayout L, float* __restrict__ grad, float* grad_out,
                                                                double* loss, double* loss_out, AdamArgs A)
 {
     __shared__ float sh[kRdSlices][32];
@@ -414,14 +419,15 @@ __global__ void __launch_bounds__(32 * kRdSlices) k_mlp_reduce(const float* __re
 #pragma unroll 8
         for (int p = slice; p < nparts; p += kRdSlices) acc += partial[(int64_t)p * L.nmaster + e];
     sh[slice][lane] = acc;
-    __syncthreads();
+    const bool failed = __syncthreads_or((int)threadIdx.x < nparts && late[threadIdx.x] != 0);
     if (slice == 0 && e < L.nmaster) {
         float g = 0.f;
 #pragma unroll
         for (int k = 0; k < kRdSlices; k++) g += sh[k][lane];
+        if (failed) g = __int_as_float(0x7fc00000);
         grad[e] = g;
         if (grad_out) grad_out[e] = g;
-        if (ADAM) {
+        if (ADAM && !failed) {
             const float mi = A.b1 * A.m[e] + (1.f - A.b1) * g;
             const float vi = A.b2 * A.v[e] + (1.f - A.b2) * g * g;
             A.m[e] = mi;
@@ -435,6 +441,7 @@ __global__ void __launch_bounds__(32 * kRdSlices) k_mlp_reduce(const float* __re
         double t = 0.0;
         for (int p = lane; p < nparts; p += 32) t += loss_part[p];
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (failed) t = __longlong_as_double(0x7ff8000000000000ll);
         if (lane == 0) {
             *loss = t;
             if (loss_out) *loss_out = t;
@@ -450,7 +457,7 @@ __global__ void k_export(const float* master, MlpLayout L, unsigned char* params
 
 template <int NOUT>
 cudaError_t train_tc(const void* X, const float* T, int64_t rows, const unsigned char* params, const MlpLayout& L,
-                     float* partial, double* loss_part, int blocks, cudaStream_t s)
+                     float* partial, double* loss_part, int* late, int blocks, cudaStream_t s)
 {
     static int attr_done[kMaxDevices] = {};  // per instantiation and device
     const int smem = (int)sizeof(TrSmem<NOUT>);
@@ -458,7 +465,7 @@ cudaError_t train_tc(const void* X, const float* T, int64_t rows, const unsigned
     if (e != cudaSuccess) return e;
     k_mlp_train_tc<NOUT><<<(unsigned)blocks, kTrThreads, smem, s>>>(reinterpret_cast<const __nv_bfloat16*>(X), T, rows,
                                                                     params, L, 1.0f / (float)(rows * L.nout), partial,
-                                                                    loss_part);
+                                                                    loss_part, late);
     return cudaGetLastError();
 }
 
@@ -476,8 +483,9 @@ cudaError_t mlp_train(unsigned char* ws, const MlpTrain& W, const void* X, const
     if (blocks > sms) blocks = sms;
     if (blocks > kMlpMaxPartials) blocks = kMlpMaxPartials;
     double* loss_part = reinterpret_cast<double*>(f + W.loss_part);
-    cudaError_t e = W.K == 16 ? train_tc<48>(X, T, rows, params, W.L, f + W.partial, loss_part, (int)blocks, s)
-                              : train_tc<24>(X, T, rows, params, W.L, f + W.partial, loss_part, (int)blocks, s);
+    int* late = reinterpret_cast<int*>(f + W.late);
+    cudaError_t e = W.K == 16 ? train_tc<48>(X, T, rows, params, W.L, f + W.partial, loss_part, late, (int)blocks, s)
+                              : train_tc<24>(X, T, rows, params, W.L, f + W.partial, loss_part, late, (int)blocks, s);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)((W.L.nmaster + 31) / 32);
     double* loss = reinterpret_cast<double*>(f + W.loss);
@@ -485,10 +493,10 @@ cudaError_t mlp_train(unsigned char* ws, const MlpTrain& W, const void* X, const
     if (adam) {
         const float b1 = 0.9f, b2 = 0.999f;
         A = {f + W.master, f + W.m, f + W.v, params, lr, b1, b2, 1e-8f, 1.f - powf(b1, (float)t), 1.f - powf(b2, (float)t)};
-        k_mlp_reduce<true><<<grid, 32 * kRdSlices, 0, s>>>(f + W.partial, loss_part, (int)blocks, W.L, f + W.grad, grad_out,
-                                                           loss, loss_out, A);
+        k_mlp_reduce<true><<<grid, 32 * kRdSlices, 0, s>>>(f + W.partial, loss_part, late, (int)blocks, W.L, f + W.grad,
+                                                           grad_out, loss, loss_out, A);
     } else {
-        k_mlp_reduce<false><<<grid, 32 * kRdSlices, 0, s>>>(f + W.partial, loss_part, (int)blocks, W.L, f + W.grad,
+        k_mlp_reduce<false><<<grid, 32 * kRdSlices, 0, s>>>(f + W.partial, loss_part, late, (int)blocks, W.L, f + W.grad,
                                                             grad_out, loss, loss_out, A);
     }
     return cudaGetLastError();
