@@ -154,47 +154,6 @@ __device__ __forceinline__ Raw zero_raw()
     return r;
 }
 
-// ---- packed FP32 -----------------------------------------------------------
-// Packed FP32 arithmetic: one instruction for two values.
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-// a - b as one packed FMA: b (-1) is exact, so this is a - b rounded once
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
-// Sums of two streams of FP32 values as unevaluated sums s + e + f: Knuth's
-// two-sum on s, its error added to e by another two-sum, that error to f.
-struct Sum3 {
-    float2 s = {0.f, 0.f}, e = {0.f, 0.f}, f = {0.f, 0.f};
-    static __device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& err)
-    {
-        const float2 t = add2(a, b), bb = sub2(t, a);
-        err = add2(sub2(a, sub2(t, bb)), sub2(b, bb));
-        return t;
-    }
-    __device__ __forceinline__ void add(float2 x)
-    {
-        float2 r;
-        s = two_sum(s, x, r);
-        e = two_sum(e, r, r);
-        f = add2(f, r);
-    }
-    // the squares: x^2 = p + r, r the rounding error of the product p (exact unless it underflows)
-    __device__ __forceinline__ void add_square(float2 x)
-    {
-        const float2 p = mul2(x, x);
-        float2 r = fma2(x, x, mul2(p, f2(-1.f)));
-        add(p);
-        e = two_sum(e, r, r);
-        f = add2(f, r);
-    }
-    __device__ __forceinline__ double value() const
-    {
-        return ((double)s.x + ((double)e.x + (double)f.x)) + ((double)s.y + ((double)e.y + (double)f.y));
-    }
-};
-
 // ---- Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11) ----------------------
 // 32-bit words throughout: the 32x32 multiplies run at the full integer rate,
 // while 64x64 products (a 64-bit variant) go through a much slower path.
@@ -266,6 +225,17 @@ __device__ __forceinline__ float recip(float x) { return fast_inverse(x); }
 // that collision), the division in FP32.
 __device__ __forceinline__ double site_inverse(double rho) { return fast_inverse(rho); }
 __device__ __forceinline__ float site_inverse(float rho) { return 1.0f / rho; }
+
+// An FP32 value in FP64 by moving its bits (the conversion instruction runs on
+// the FP64 pipe, two lanes a clock); zeros, subnormals, infinities and NaN
+// through the conversion itself.
+__device__ __forceinline__ double widen(float v)
+{
+    const uint32_t b = __float_as_uint(v);
+    if ((b << 1) - 0x01000000u >= 0xfe000000u) return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
 
 __device__ __forceinline__ int wrapi(int v, int E) { return v < 0 ? v + E : (v >= E ? v - E : v); }
 

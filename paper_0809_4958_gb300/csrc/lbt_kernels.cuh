@@ -1939,6 +1939,29 @@ __global__ void k_read_dev(const typename Stor<ST>::E* Ab, int64_t count, typena
 constexpr int kConsThreads = 128;
 constexpr int kConsSitesPerThread = kConsChunk / kConsThreads;
 
+// Sums of two streams of FP32 values as unevaluated sums s + e + f: Knuth's
+// two-sum on s, its error added to e by another two-sum, that error to f.
+struct Sum3 {
+    float2 s = {0.f, 0.f}, e = {0.f, 0.f}, f = {0.f, 0.f};
+    static __device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& err)
+    {
+        const float2 t = add2(a, b), bb = sub2(t, a);
+        err = add2(sub2(a, sub2(t, bb)), sub2(b, bb));
+        return t;
+    }
+    __device__ __forceinline__ void add(float2 x)
+    {
+        float2 r;
+        s = two_sum(s, x, r);
+        e = two_sum(e, r, r);
+        f = add2(f, r);
+    }
+    __device__ __forceinline__ double value() const
+    {
+        return ((double)s.x + ((double)e.x + (double)f.x)) + ((double)s.y + ((double)e.y + (double)f.y));
+    }
+};
+
 // Sums over this thread's sites of a chunk in FP64 (every format; the reduced
 // ones only where a value is not finite or so large that FP32 overflows).
 template <int ST>

@@ -156,10 +156,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     float colsum[OH];  // this thread's share of sum_r dY[r][o], FP32
 #pragma unroll
     for (int c = 0; c < OH; c++) colsum[c] = 0.f;
-    // sum of the squares of Y - T: FP32 triple words, no less exact than an FP64 sum (Sum3); what their range does not
-    // hold goes to an FP64 one
-    Sum3 sq;
-    double sq_far = 0.0;
+    double sq = 0.0;  // sum of the squares of Y - T
     uint32_t phase = 0;
     bool ok = true, first = true;
     const bool t_vec = (reinterpret_cast<uintptr_t>(T) & 15) == 0;
@@ -181,6 +178,18 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         return ok;
     };
 
+    float t[OH];  // targets, then Y - T
+    // a third of the row's squares: an FP64 instruction of a warp takes its quarter of the SM 64 cycles, so they go
+    // where the block waits for an MMA anyway (as FP32 triple words behind the first of them: 4 us a tile)
+    auto add_squares = [&](int third) {
+#pragma unroll
+        for (int c = 0; c < OH; c++)
+            if (c * 3 / OH == third) {
+                const double d = widen(t[c]);
+                sq = fma(d, d, sq);
+            }
+    };
+
     const int64_t ntiles = (rows + kTcRows - 1) / kTcRows;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t r = tile * kTcRows + m;
@@ -196,7 +205,6 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                 *reinterpret_cast<uint4*>(sm.x + core_off(m, 8 * (2 * half + c), kMlpIn)) = v;
             }
         }
-        float t[OH];
         {
             const float* tr = T + (in ? r : 0) * NOUT + half * OH;
 #pragma unroll
@@ -280,20 +288,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             mma_chain<kTcRows / 16>(tmem + kColW3, a2, 2 * kR128, kR128, kCore, ay, 2 * kRNP, kRNP, kCore,
                                     tc_idesc(kMlpHidden, NP, true, true), !first);
         }
-        // the loss, meanwhile: squares of 24-bit values are exact in two words from 2^-51 on, and far from overflow below 2^50
-#pragma unroll
-        for (int c = 0; c < OH; c += 2) {
-            float d[2];
-#pragma unroll
-            for (int k = 0; k < 2; k++) {
-                d[k] = t[c + k];
-                if (!(fabsf(d[k]) >= 0x1p-51f && fabsf(d[k]) < 0x1p50f)) {
-                    if (d[k] != 0.f) sq_far += (double)d[k] * (double)d[k];
-                    d[k] = 0.f;
-                }
-            }
-            sq.add_square(make_float2(d[0], d[1]));
-        }
+        add_squares(0);
         if (!wait_mma()) break;
         masked_epilogue(trow + kColWork + half * kTrHalf, sm.h2, sm.dz2, m, half * kTrHalf);
         issue_fence();
@@ -308,6 +303,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             mma_chain<kTcRows / 16>(tmem + kColB2, az2, 2 * kR128, kR128, kCore, aone, 2 * kR16, kR16, kCore,
                                     tc_idesc(kMlpHidden, 16, true, true), !first);
         }
+        add_squares(1);
         if (!wait_mma()) break;
         masked_epilogue(trow + kColWork + half * kTrHalf, sm.h1, sm.h2, m, half * kTrHalf);
         issue_fence();
@@ -320,6 +316,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             tc_commit(&sm.bar);
         }
         first = false;
+        add_squares(2);
         if (!wait_mma()) break;  // every operand read: the next tile may be staged
     }
     if (!ok) tc_wait(&sm.bar, phase ^ 1u);  // let an MMA still in flight finish (bounded); `late` below says what happened
@@ -359,7 +356,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         for (int o = 16; o > 0; o >>= 1) colsum[c] += __shfl_xor_sync(0xffffffffu, colsum[c], o);
         if (lane == 0) sm.col[q][half * OH + c] = colsum[c];
     }
-    double loss = sq.value() + sq_far;
+    double loss = sq;
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
     if (lane == 0) sm.loss[warp] = loss;
     tc_fence_before();

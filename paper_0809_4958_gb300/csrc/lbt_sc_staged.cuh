@@ -371,6 +371,14 @@ __device__ __forceinline__ void staged_tile(const SCParams& p, const StagedTile<
 }
 
 // ---- two adjacent sites per consumer thread (FP32 and 16-bit storage) -----
+// Packed FP32 arithmetic: one instruction advances both sites of a thread.
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+// a - b as one packed FMA: b (-1) is exact, so this is a - b rounded once
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
 // Loads and stores of a pair of adjacent stored elements: one aligned word
 // for the pair of a thread (elements e, e + 1 with e even), two scalar loads
 // for the x-shifted pairs, conversions to and from FP32 packed where the

@@ -194,17 +194,6 @@ __device__ double block_sum(double v, double* sh)
     return t;
 }
 
-// An FP32 value in FP64 by moving its bits (the conversion instruction runs on
-// the FP64 pipe, two lanes a clock); zeros, subnormals, infinities and NaN
-// through the conversion itself.
-__device__ __forceinline__ double widen(float v)
-{
-    const uint32_t b = __float_as_uint(v);
-    if ((b << 1) - 0x01000000u >= 0xfe000000u) return (double)v;
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double v) { return v; }
-
 // sqrt(x) by Goldschmidt's iteration from an FP32 start: two steps from 22
 // bits (x outside the FP32 range, zero, infinite or NaN: the library's).
 __device__ __forceinline__ double quick_sqrt(double x)
