@@ -3,6 +3,7 @@
 // Host-side bookkeeping only: arena layout, box and chain tables, the ring of
 // coarse boundary samples, step ordering and launches.  All arithmetic of the
 // method runs in the kernels of lbt_kernels.cuh and lbt_synth.cu.
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -214,6 +215,7 @@ struct lb_ctx {
     std::vector<int64_t> tile_prefix;  // for the current block size
     std::mutex host_mutex;
     std::vector<double*> host_slots, host_free;  // pinned (host_mutex): every slot, and those no call holds (HostSlot)
+    std::atomic<bool> copy_behind{false};  // an lb_sync that timed out left its copy on the stream
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
     bool graph_parity = true;
@@ -1042,9 +1044,20 @@ int32_t lb_vorticity(lb_ctx* ctx, int32_t box, int32_t lo, int32_t hi, double* o
 int32_t lb_sync(lb_ctx* ctx, int32_t timeout_ms)
 {
     if (!ctx) return LB_ERR_ARG;
+    // The copy of the status goes ahead of the wait, so that one wait covers
+    // both; a caller that polls a busy stream leaves one such copy behind, not
+    // one a poll (about a thousand fill the stream's queue, and the next call
+    // then waits for a place in it, whatever its timeout).
+    int st = LB_OK;
+    if (ctx->copy_behind.load()) {
+        st = wait_stream(ctx, timeout_ms);
+        if (st) return st;
+        ctx->copy_behind.store(false);
+    }
     const HostSlot host(ctx);
-    int st = copy_status(ctx, host);
+    st = copy_status(ctx, host);
     if (!st) st = wait_stream(ctx, timeout_ms);
+    if (st == LB_ERR_TIMEOUT) ctx->copy_behind.store(true);
     if (st) return st;
     return first_status(ctx, host, -1);
 }
