@@ -396,10 +396,20 @@ int enqueue_step(lb_ctx* ctx, int64_t n)
     sp.wait_ns = ctx->wait_ns;
     sp.withhold_tile = ctx->inject == LB_INJECT_WITHHOLD_LAST_TILE ? sp.total_tiles - 1 : -1;
     sp.hint_loads = nch > 0;
-    // several boxes: runs of four neighbouring tiles where every SM takes more
-    // than 64, so that a producer meets a new box every fourth tile
-    sp.claim = ctx->nboxes > 1 && ctx->sms > 0 && sp.total_tiles > 64 * (int64_t)ctx->sms ? 4 : 1;
-    sp.pad_claim = 0;
+    // Several boxes: a producer that meets a new box with nearly every tile does not keep its consumers fed, so it claims
+    // runs of neighbouring tiles where an SM takes several runs (or their tail costs more) and boxes are small enough for
+    // it to matter.  Not in FP64, where a tile's arithmetic takes longer than the producer (80 boxes of 32^3: 728 us a
+    // step, 781 in runs of four).  FP32 / binary16, single tiles -> runs: 24 boxes of 32^3 with 16 beads (5.5 tiles to an
+    // SM) 52 -> 49 / 49 -> 44 us, 96 with 32 beads (22) 139 -> 116 / 124 -> 93, 40 of 48^3 with 64 beads (31) 173 -> 140 /
+    // 154 -> 106, 320 of 32^3 without beads (74) 353 -> 254 / 294 -> 180; 12 boxes of 32^3 (2.8) 20.1 / 17.4 against
+    // 21.2 / 18.2 in runs of two, two boxes of 128^3 (29) 100 against 105.
+    const int64_t per_sm = ctx->sms > 0 ? sp.total_tiles / ctx->sms : 0;
+    const int64_t per_box_sms = sp.total_tiles / ((int64_t)ctx->nboxes * (ctx->sms > 0 ? ctx->sms : 1));  // tiles of a box, in SMs
+    sp.claim = 1;
+    if (ctx->storage != kF64 && ctx->nboxes > 1) {
+        if (per_sm >= 16 && per_box_sms < 4) sp.claim = 4;
+        else if (per_sm >= 4 && per_box_sms < 1) sp.claim = 2;
+    }
     sp.ends_step = nch == 0 && ctx->kernel == LB_KERNEL_STAGED;
     const bool timed = ctx->profiling && ctx->prof_used + 2 <= ctx->prof_ev.size();
     // inside a stream capture the timing events must become event-record nodes of the graph

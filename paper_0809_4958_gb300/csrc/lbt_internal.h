@@ -166,7 +166,6 @@ struct SCParams {
     int64_t withhold_tile;        // test only: the staged producer never arms this tile (-1: none)
     int32_t hint_loads;           // 1: the staged bulk copies take the L2 evict-first policy (chains in the launch)
     int32_t claim;                // neighbouring tiles the staged producer claims at once
-    int32_t pad_claim;
     int32_t ends_step;            // 1: no chain in the launch, the staged kernel advances the step and resets the counter
 };
 
