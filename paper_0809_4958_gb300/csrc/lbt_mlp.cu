@@ -140,11 +140,13 @@ __global__ void __launch_bounds__(32 * kTgtWarps) k_mlp_targets(const R* s_prev,
                                                                 float inv_umax, float* T)
 {
     __shared__ float sh[kTgtRows][3 * kTgtSub + 1];
-    const int fe = E * E, rows = 6 * fe;
+    const int64_t fe = (int64_t)E * E, rows = 6 * fe;  // beyond 32 bits from E = 18919 on
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r_blk = blockIdx.x * kTgtRows, r = r_blk + lane;
+    const int64_t r_blk = (int64_t)blockIdx.x * kTgtRows, r = r_blk + lane;
     const bool in = r < rows;
-    const int f = in ? r / fe : 0, site = in ? r - f * fe : 0;
+    int f = 0;  // the row's face (by comparisons: a 64-bit division is a long instruction sequence)
+    for (int k = 1; k < 6; k++) f += in && r >= k * fe;
+    const int64_t site = in ? r - f * fe : 0;
     float u0[3], u1[3], u2[3], m0[3];
     for (int c = 0; c < 3; c++) {
         const int64_t o = (int64_t)(f * 3 + c) * fe + site;
@@ -168,10 +170,10 @@ __global__ void __launch_bounds__(32 * kTgtWarps) k_mlp_targets(const R* s_prev,
             }
         }
         __syncthreads();
-        const int w = 3 * ns, nr = min(kTgtRows, rows - r_blk);
+        const int w = 3 * ns, nr = (int)min((int64_t)kTgtRows, rows - r_blk);
         for (int e = threadIdx.x; e < nr * w; e += blockDim.x) {
             const int rr = e / w, c = e - rr * w;
-            T[(int64_t)(r_blk + rr) * 3 * K + 3 * sb + c] = sh[rr][c];
+            T[(r_blk + rr) * 3 * K + 3 * sb + c] = sh[rr][c];
         }
         __syncthreads();
     }
