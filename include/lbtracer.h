@@ -325,7 +325,8 @@ int64_t lb_current_step(const lb_ctx* ctx);
  *   warp, 15 consumer warps), tiles of 480 x sites_per_thread sites staged
  *   in as many pipeline stages as fit in shared memory; threads must be 0;
  *   sites_per_thread 0 (default: 1 for FP64, 2 otherwise), 1, or 2 (not
- *   FP64); ctas = persistent grid (0 = one block per SM).
+ *   FP64); ctas = persistent grid (0 = one block per SM; a larger one is
+ *   accepted and runs as one block per SM, which a block fills).
  *   kernel LB_KERNEL_REGISTER: threads per block (multiple of 32, 64 .. 256),
  *   ctas = persistent grid (0 = one block per tile), sites_per_thread
  *   (0 = default: 2 for FP64, 4 for FP32, 8 for 16-bit storage; half or a
@@ -344,8 +345,8 @@ int32_t lb_set_launch(lb_ctx* ctx, int32_t kernel, int32_t threads, int32_t ctas
  *   slot masked rather than branched; in FP64 storage it gives chains of up
  *   to 128 beads four warps to 32 beads instead, split by the kind of pair and
  *   then by component.  One barrier over the MD threads per substep (two in
- *   the FP64 split).  lanes x ceil(largest chain / beads_per_thread) <= 512.  Used by the autotuner; drops a captured graph.  LB_ERR_ARG
- *   otherwise. */
+ *   the FP64 split).  lanes x ceil(largest chain / beads_per_thread) <= 512.
+ *   Used by the autotuner; drops a captured graph.  LB_ERR_ARG otherwise. */
 int32_t lb_set_bead_launch(lb_ctx* ctx, int32_t lanes, int32_t beads_per_thread);
 
 /*

@@ -2216,7 +2216,7 @@ cudaError_t Launch<ST>::fields(const void* A, const BoxDev* boxes, int box, int6
 {
     // 16-byte loads; a row takes at least two groups (the two x faces lie in
     // different ones), so 16-bit storage at E = 8 takes 8-byte loads
-        constexpr int VW = 16 / (int)sizeof(typename Stor<ST>::E);
+    constexpr int VW = 16 / (int)sizeof(typename Stor<ST>::E);
     if constexpr (VW == 8)
         if (boxes[box].E < 2 * VW) return launch_fields<ST, VW / 2>(A, boxes[box], what, dst, s);
     return launch_fields<ST, VW>(A, boxes[box], what, dst, s);

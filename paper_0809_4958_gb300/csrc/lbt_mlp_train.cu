@@ -13,8 +13,8 @@
 // What bounds it: latency.  A tile is a chain of six products, each an MMA, a
 // commit, a wait and an epilogue, about 2 us in all, and the 16384 rows of the
 // benchmark are 128 tiles, fewer than SMs; its 2.5 GFLOP would take 1.3 us and
-// its bytes less.  One training step of 16384 rows (K = 16): 19.0 us for this
-// kernel, 4.3 us for the reduction with Adam.  As a chain of twelve launches
+// its bytes less.  One training step of 16384 rows (K = 16): 26.0 us, a sixth
+// of it the reduction with Adam.  As a chain of twelve launches
 // (forward, loss, three weight and two activation gradients that staged their
 // operands transposed, three column sums, Adam, export) through global memory
 // it took 240 us.  Eight warps, two to a TMEM quadrant, halve the epilogues.

@@ -1082,11 +1082,17 @@ __device__ __forceinline__ void prefetch_mlp_residuals(const SCParams& p, const 
 // sample k / 6 of those with a weight, then the upsampler's residuals of the
 // substep; face (k % 6) / 3, component k % 3.  Runs are `stride` elements long,
 // start at a multiple of four (16 bytes) and lie inside E^2, itself a multiple
-// of 64.  Boxes whose runs do not fit the room of a stage (short rows, many
-// samples) load from global memory.  Fills the header's fields; returns the
-// run's base (null: none), E^2 - stride in last_start.  (With the producer's
-// work per box: 128 boxes of 64^3 with the upsampler 1198 -> 846 us a step, 512
-// uneven boxes with chains 1817 -> 1496.)
+// of 64.  Fills the header's fields; returns the run's base (null: none),
+// E^2 - stride in last_start.
+//
+// Boxes whose runs do not fit the room of a stage load from global memory.  In
+// FP32 (2544 bytes) two samples, linear in time, fit from E = 24 on, Hermite's
+// four from 48, and with the upsampler's residual from 64 (2400 bytes there,
+// 2880 at 56); in 16-bit storage (960 bytes) two samples fit from 64, four, also
+// with the residual, from 240.  Staged against loaded, us a step: FP32 linear 128
+// boxes of 64^3 747 / 798, 512 of 32^3 418 / 453, one of 128^3 53.4 / 54.2; with the
+// upsampler 128 of 64^3 849 / 889; binary16 linear 128 of 64^3 528 / 537, one of
+// 256^3, where one site in 128 is on an x face, 232 / 224.
 template <int ROOM, int ST>
 __device__ __forceinline__ const float* edge_runs(const SCParams& p, StagedTile<ST>& th, int T, int lane, int& last_start)
 {
